@@ -16,6 +16,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
+
 #include "celeris_gb.h"
 
 namespace cel {
@@ -68,6 +70,15 @@ struct Coef {
     real g, eps, theta, ws, dt, Bd, B3, sixth;
     real rdx, rdy, hrdx, hrdy, rdx2, rdy2, rdxdy4, rdx3h, rdy3h, rdxdy2h, rdx2dyh;
     real fric;           // quadratic f, or g n^2 for Manning
+    // constants of the stencil's per-cell expressions, each rounded once:
+    real th2;            // 2 theta (slopes before their factor 1/4)
+    real hwet;           // eps^(1/4): the depth from which Eq. 14's factor is 1/h
+    real hgx, hgy;       // g / (2 dx), g / (2 dy) (bed slope from corner sums)
+    real Bdg;            // B g
+    real c6;             // 1 / (24 dx dy) (first-derivative products of F*, G*)
+    real B3xy;           // (B + 1/3) / (4 dx dy) (mixed derivatives of F*, G*)
+    real ab[3];          // 23, -16, 5 dt / 12 (Eq. 15)
+    real am[4];          // 9, 19, -5, 1 dt / 24 (Eq. 18)
     int spw[4];          // sponge width in cells per side (0: not a sponge)
     int sine;            // bit s set: side s is a sine maker
     int npos;            // positions per side in the ghost table
@@ -98,6 +109,20 @@ inline Coef<real> make_coef(const Geo &G, const Phys &p, const Bnd &b)
     c.rdxdy2h = real(1.0 / (2.0 * G.dx * G.dy * G.dy));
     c.rdx2dyh = real(1.0 / (2.0 * G.dx * G.dx * G.dy));
     c.fric = real(p.friction == kFricManning ? p.g * p.fcoef * p.fcoef : p.fcoef);
+    c.th2 = real(2.0 * p.theta);
+    c.hwet = real(std::sqrt(std::sqrt(p.eps)));
+    c.hgx = real(0.5 * p.g / G.dx);
+    c.hgy = real(0.5 * p.g / G.dy);
+    c.Bdg = real(p.Bd * p.g);
+    c.c6 = real(1.0 / (24.0 * G.dx * G.dy));
+    c.B3xy = real((p.Bd + 1.0 / 3.0) / (4.0 * G.dx * G.dy));
+    c.ab[0] = real(23.0 * p.dt / 12.0);
+    c.ab[1] = real(-16.0 * p.dt / 12.0);
+    c.ab[2] = real(5.0 * p.dt / 12.0);
+    c.am[0] = real(9.0 * p.dt / 24.0);
+    c.am[1] = real(19.0 * p.dt / 24.0);
+    c.am[2] = real(-5.0 * p.dt / 24.0);
+    c.am[3] = real(p.dt / 24.0);
     c.sine = 0;
     for (int s = 0; s < 4; s++) {
         c.spw[s] = b.s[s].type == kSponge ? b.s[s].width : 0;

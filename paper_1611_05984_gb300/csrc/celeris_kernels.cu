@@ -399,22 +399,6 @@ struct StencilSmem {
     uint32_t colbits[kTile];
 };
 
-// Update of one unknown (w, U* or V*) with right side R and mixed term Phi
-// (0 for w), Sec. 2.3, returned as the increment X^{n+1} - X^n.  Carries
-// (per cell, row-major):
-//   a = -16 (dt/12) R^{n-1} - 3 Phi^{n-1}       (in place)
-//   b = 5 (dt/12) R^{n-2} + Phi^{n-2}           (two slots, by step parity)
-// so that Eq. 15-17 read X^{n+1} - X^n = 23 (dt/12) R^n + 2 Phi^n + a + b.
-// The first two steps are forward Euler; the second adds Phi^1 - Phi^0,
-// for which `a` holds Phi^0 after the first.  With K > 0 also
-//   q = (dt/24)(-5 R^{n-1} + R^{n-2}),  e = (dt/24) R^{n-1},
-//   Y = X0 + 19 (dt/24) R^n - Phi^n + q         (corrector base),
-// so that Eq. 18-20 read X^{n+1} - X0 = Y - X0 + 9 (dt/24) R^{n+1} + Phi^{n+1}
-// (the AM4 stage returns Y + 9 (dt/24) R + Phi).  For w, X0 = w^n, so the
-// corrector returns w^{n+1} itself.  U* and V* are carried as increments
-// only (X0 = 0): the line solves find P^{n+1} - P^n from the increment of U*,
-// which equals recomputing U*^n from P^n by Eq. 23 but keeps the rounding
-// relative to the increment instead of to P.
 // History of one unknown (w, U* or V*) for the update of Sec. 2.3, with R
 // its right side and Phi its mixed term (0 for w); the AB3 and AM4 stages
 // return the increment X^{n+1} - X^n (for the AM4 stage of w: w^{n+1}).
@@ -491,17 +475,19 @@ __device__ __forceinline__ real advance(const StencilArgs<real> &A, int v, real 
 {
     const int kind = stage_kind<kSpec>(A);
     const bool ring = stage_ring<kSpec>(A);
-    const real dt = A.c.dt, c12 = dt / real(12), c24 = dt / real(24);
-    if (kind == kAM4) return c.Y + real(9) * c24 * R + Phi;
+    const Coef<real> &C = A.c;
+    if (kind == kAM4) return c.Y + C.am[0] * R + Phi;
     if (ring) {
         real D;
         if (kind == kEuler0) {
-            D = dt * R;
+            D = C.dt * R;
         } else if (kind == kEuler1) {
-            D = dt * R + (Phi - c.p1);
+            D = C.dt * R + (Phi - c.p1);
         } else {
-            D = c12 * (real(23) * R - real(16) * c.r1 + real(5) * c.r2) + real(2) * Phi - real(3) * c.p1 + c.p2;
-            A.Y[v][k] = X0 + c24 * (real(19) * R - real(5) * c.r1 + c.r2) - Phi;
+            D = C.ab[0] * R + C.ab[1] * c.r1 + C.ab[2] * c.r2;
+            if (v > 0) D += real(2) * Phi - real(3) * c.p1 + c.p2;
+            const real y = X0 + (C.am[1] * R + C.am[2] * c.r1 + C.am[3] * c.r2);
+            A.Y[v][k] = v > 0 ? y - Phi : y;
         }
         A.R0[v][k] = R;
         if (v > 0) A.F0[v][k] = Phi;
@@ -509,16 +495,16 @@ __device__ __forceinline__ real advance(const StencilArgs<real> &A, int v, real 
     }
     real D;
     if (kind == kEuler0) {
-        D = dt * R;
+        D = C.dt * R;
         A.a[v][k] = Phi;
     } else if (kind == kEuler1) {
-        D = dt * R + (Phi - c.a);
-        A.a[v][k] = real(-16) * c12 * R - real(3) * Phi;
+        D = C.dt * R + (Phi - c.a);
+        A.a[v][k] = C.ab[1] * R - real(3) * Phi;
     } else {
-        D = real(23) * c12 * R + real(2) * Phi + (c.a + c.b);
-        A.a[v][k] = real(-16) * c12 * R - real(3) * Phi;
+        D = C.ab[0] * R + real(2) * Phi + (c.a + c.b);
+        A.a[v][k] = C.ab[1] * R - real(3) * Phi;
     }
-    A.b[v][k] = real(5) * c12 * R + Phi;
+    A.b[v][k] = C.ab[2] * R + Phi;
     return D;
 }
 
@@ -616,6 +602,48 @@ struct SharedOrigin {
     __device__ __forceinline__ int y0() const { return ld(1); }
 };
 
+// Fluxes through faces f0 .. f1 - 1 of one row (kX: x-faces, r the row) or
+// one column (y-faces, r the column) of the staged tile.
+template <typename real, bool kX>
+__device__ __forceinline__ void sweep_faces(StencilSmem<real> &sm, const Coef<real> &C, int r, int f0, int f1)
+{
+    // strides along the sweep, and from a face's first corner to its second
+    constexpr int sq = kX ? 1 : kStride, sc = kX ? 1 : kCornerStride, sc2 = kX ? kCornerStride : 1;
+    constexpr int sf = kX ? 1 : kTile, sv = kX ? kTile * (kTile + 1) : (kTile + 1) * kTile;
+    const int o0 = (kX ? (r + kHalo) * kStride : r + kHalo) + f0 * sq;   // cell f0 - 2
+    const real *pw = sm.w + o0, *pn = (kX ? sm.P : sm.Q) + o0, *pt = (kX ? sm.Q : sm.P) + o0;
+    const real *cb = sm.Bc + (kX ? (r + 1) * kCornerStride : r + 1) + f0 * sc;   // face f0 - 1
+    real *out = (kX ? &sm.Fx[0][r][0] : &sm.Fy[0][0][r]) + f0 * sf;
+    FaceSweep<real> sweep;
+    real lo[3], hi[3], hn[3], dlo, dhi, dn;
+    const real c0[3] = {pw[0], pn[0], pt[0]}, c1[3] = {pw[sq], pn[sq], pt[sq]};
+    sweep.open(C.th2, c0, c1);
+    real Bf = half_r(cb[sc] + cb[sc + sc2]);   // bed at the face about to be computed
+    {
+        const real q[3] = {pw[2 * sq], pn[2 * sq], pt[2 * sq]};
+        sweep.next(C.th2, q, half_r(cb[0] + cb[sc2]), Bf, lo, hi, dlo, dhi);
+    }
+    for (int f = f0; f < f1; f++) {
+        pw += sq;
+        pn += sq;
+        pt += sq;
+        cb += sc;
+        const real Bn = half_r(cb[sc] + cb[sc + sc2]);
+        const real q[3] = {pw[2 * sq], pn[2 * sq], pt[2 * sq]};
+        sweep.next(C.th2, q, Bf, Bn, lo, hn, dlo, dn);
+        real H[3];
+        face_flux_step(C.g, C.eps, C.hwet, hi[0], hi[1], hi[2], dhi, lo[0], lo[1], lo[2], dlo, H);
+        out[0] = H[0];
+        out[kX ? sv : 2 * sv] = H[1];   // momentum normal to the face
+        out[kX ? 2 * sv : sv] = H[2];
+        out += sf;
+#pragma unroll
+        for (int v = 0; v < 3; v++) hi[v] = hn[v];
+        dhi = dn;
+        Bf = Bn;
+    }
+}
+
 // One 32 x 32 tile of one grid, at the origin O gives: the whole stencil stage.
 template <typename real, int kSpec, typename Origin>
 __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const Origin &O, unsigned char *smem_raw)
@@ -626,7 +654,6 @@ __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const O
     const int tid = threadIdx.x;
     const Coef<real> &C = A.c;
     const real ws = C.ws, g = C.g, eps = C.eps;
-    const real th = C.theta;
 
     // ---- 1. stage the state tile (+2 halo) and the bed corners; Q is
     //         column-major, so its tile is staged along y and transposed.
@@ -720,6 +747,11 @@ __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const O
     {
         const int lane = tid & 31, wq = (tid >> 5) & 3;
         const int f0 = wq * 8, f1 = wq == 3 ? kTile + 1 : f0 + 8;
+        if constexpr (sizeof(real) == 8) {
+        if (tid < 4 * 32) sweep_faces<real, true>(sm, C, lane, f0, f1);
+        else sweep_faces<real, false>(sm, C, lane, f0, f1);
+        } else {
+        const real th = C.theta;
         real lo[3], hiL[3], hiR[3];
         // the three cells a reconstruction reads slide along the row (or
         // column) one cell per face, so each face loads one new cell and one
@@ -806,14 +838,12 @@ __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const O
                 Bf = Bn;
             }
         }
+        }
     }
     __syncthreads();
 
     // ---- 5. per cell: Eq. 9-13, friction, U*, V*, update
-    const real dt = C.dt;
-    const real rdx = C.rdx, rdy = C.rdy, rdx2 = C.rdx2, rdy2 = C.rdy2, rdxdy4 = C.rdxdy4;
-    const real rdx3h = C.rdx3h, rdy3h = C.rdy3h, rdxdy2h = C.rdxdy2h, rdx2dyh = C.rdx2dyh;
-    const real Bd = C.Bd, B3 = C.B3, sixth = C.sixth;
+    const real rdx = C.rdx, rdy = C.rdy;
     const bool bsnq = A.phy.model == kBsnq;
     const int friction = A.phy.friction;
     const int lane = tid & 31;
@@ -840,52 +870,51 @@ __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const O
         }
         const real *cb = sm.Bc + (cy + 1) * kCornerStride + cx + 1;
         real c00 = cb[0], c10 = cb[1], c01 = cb[kCornerStride], c11 = cb[kCornerStride + 1];
-        real Bb = cell_bbar(c00, c10, c01, c11);
-        real BxW = real(0.5) * (c00 + c01), BxE = real(0.5) * (c10 + c11);
-        real ByS = real(0.5) * (c00 + c10), ByN = real(0.5) * (c01 + c11);
+        const real Bb = cell_bbar(c00, c10, c01, c11);
         real w0 = sm.w[o], P0 = sm.P[o], Q0 = sm.Q[o];
-        real hb = w0 - Bb;
-        real E = -(sm.Fx[0][cy][cx + 1] - sm.Fx[0][cy][cx]) * rdx - (sm.Fy[0][cy + 1][cx] - sm.Fy[0][cy][cx]) * rdy;
-        real F = -(sm.Fx[1][cy][cx + 1] - sm.Fx[1][cy][cx]) * rdx - (sm.Fy[1][cy + 1][cx] - sm.Fy[1][cy][cx]) * rdy -
-                 g * hb * (BxE - BxW) * rdx;
-        real Gq = -(sm.Fx[2][cy][cx + 1] - sm.Fx[2][cy][cx]) * rdx - (sm.Fy[2][cy + 1][cx] - sm.Fy[2][cy][cx]) * rdy -
-                  g * hb * (ByN - ByS) * rdy;
+        const real hb = w0 - Bb;
+        const real E = (sm.Fx[0][cy][cx] - sm.Fx[0][cy][cx + 1]) * rdx + (sm.Fy[0][cy][cx] - sm.Fy[0][cy + 1][cx]) * rdy;
+        real F = (sm.Fx[1][cy][cx] - sm.Fx[1][cy][cx + 1]) * rdx + (sm.Fy[1][cy][cx] - sm.Fy[1][cy + 1][cx]) * rdy;
+        real Gq = (sm.Fx[2][cy][cx] - sm.Fx[2][cy][cx + 1]) * rdx + (sm.Fy[2][cy][cx] - sm.Fy[2][cy + 1][cx]) * rdy;
+        // bed slope: the face beds' difference is half that of the corner sums
+        F -= hb * C.hgx * ((c10 + c11) - (c00 + c01));
+        Gq -= hb * C.hgy * ((c01 + c11) - (c00 + c10));
         if (friction != kFricNone) {   // Eq. 31-32 with the Eq. 14 device
-            real hinv = desing(fmax(hb, real(0)), eps);
-            real fc = friction == kFricManning ? C.fric * cbrt_r(hinv) : C.fric;
-            real mag = sqrt(P0 * P0 + Q0 * Q0);
-            F -= fc * P0 * mag * hinv * hinv;
-            Gq -= fc * Q0 * mag * hinv * hinv;
+            const real fm = friction_depth(friction, C.fric, hb, eps, C.hwet) * sqrt_r(P0 * P0 + Q0 * Q0);
+            F -= fm * P0;
+            Gq -= fm * Q0;
         }
         real Fs = real(0), Gs = real(0);
         const int od = (cy + 1) * kDStride + cx + 1;
         const real dd = sm.d[od];
         if (bsnq) {
-            const real ddx = (sm.d[od + 1] - sm.d[od - 1]) * C.hrdx;
-            const real ddy = (sm.d[od + kDStride] - sm.d[od - kDStride]) * C.hrdy;
+            const real dDx = sm.d[od + 1] - sm.d[od - 1], dDy = sm.d[od + kDStride] - sm.d[od - kDStride];
+            const real d2 = dd * dd;
             const real *W = sm.w + o;
             const int S1 = kStride, S2 = 2 * kStride;
             // eta = w - w_s enters only through differences, where w_s cancels
-            real e00 = W[0];
-            real eE = W[1], eW = W[-1], eN = W[S1], eS = W[-S1];
-            real eEE = W[2], eWW = W[-2], eNN = W[S2], eSS = W[-S2];
-            real eNE = W[S1 + 1], eNW = W[S1 - 1], eSE = W[-S1 + 1], eSW = W[-S1 - 1];
-            real exx = (eE - real(2) * e00 + eW) * rdx2;
-            real eyy = (eN - real(2) * e00 + eS) * rdy2;
-            real exy = (eNE - eSE - eNW + eSW) * rdxdy4;
-            real exxx = (eEE - real(2) * eE + real(2) * eW - eWW) * rdx3h;
-            real eyyy = (eNN - real(2) * eN + real(2) * eS - eSS) * rdy3h;
-            real exyy = ((eNE - real(2) * eE + eSE) - (eNW - real(2) * eW + eSW)) * rdxdy2h;
-            real exxy = ((eNE - real(2) * eN + eNW) - (eSE - real(2) * eS + eSW)) * rdx2dyh;
-            F += Bd * g * dd * dd * dd * (exxx + exyy) + Bd * g * dd * dd * (ddx * (real(2) * exx + eyy) + ddy * exy);
-            Gq += Bd * g * dd * dd * dd * (eyyy + exxy) + Bd * g * dd * dd * (ddy * (real(2) * eyy + exx) + ddx * exy);
+            const real e00 = w0;
+            const real eE = W[1], eW = W[-1], eN = W[S1], eS = W[-S1];
+            const real eNE = W[S1 + 1], eNW = W[S1 - 1], eSE = W[-S1 + 1], eSW = W[-S1 - 1];
+            const real pN = eNE - eNW, pS = eSE - eSW;             // x-differences of the rows above and below
+            const real gx = eE - eW, gy = eN - eS;
+            const real exy = (pN - pS) * C.rdxdy4;
+            const real exx = (eE - real(2) * e00 + eW) * C.rdx2;
+            const real eyy = (eN - real(2) * e00 + eS) * C.rdy2;
+            const real exxx = (W[2] - W[-2]) - real(2) * gx;
+            const real eyyy = (W[S2] - W[-S2]) - real(2) * gy;
+            const real exyy = (pN + pS) - real(2) * gx;
+            const real exxy = ((eNE - eSE) + (eNW - eSW)) - real(2) * gy;
+            const real ddx = dDx * C.hrdx, ddy = dDy * C.hrdy;
+            const real K2 = C.Bdg * d2;
+            F += K2 * (dd * (exxx * C.rdx3h + exyy * C.rdxdy2h) + ddx * (real(2) * exx + eyy) + ddy * exy);
+            Gq += K2 * (dd * (eyyy * C.rdy3h + exxy * C.rdx2dyh) + ddy * (real(2) * eyy + exx) + ddx * exy);
             const real *Pt = sm.P + o, *Qt = sm.Q + o;
-            real Qx = (Qt[1] - Qt[-1]) * C.hrdx, Qy = (Qt[S1] - Qt[-S1]) * C.hrdy;
-            real Qxy = (Qt[S1 + 1] - Qt[-S1 + 1] - Qt[S1 - 1] + Qt[-S1 - 1]) * rdxdy4;
-            real Px = (Pt[1] - Pt[-1]) * C.hrdx, Py = (Pt[S1] - Pt[-S1]) * C.hrdy;
-            real Pxy = (Pt[S1 + 1] - Pt[-S1 + 1] - Pt[S1 - 1] + Pt[-S1 - 1]) * rdxdy4;
-            Fs = dd * ddx * Qy * sixth + dd * ddy * Qx * sixth + B3 * dd * dd * Qxy;
-            Gs = dd * ddy * Px * sixth + dd * ddx * Py * sixth + B3 * dd * dd * Pxy;
+            const real m1 = dd * dDx * C.c6, m2 = dd * dDy * C.c6, m3 = C.B3xy * d2;
+            Fs = m1 * (Qt[S1] - Qt[-S1]) + m2 * (Qt[1] - Qt[-1]) +
+                 m3 * ((Qt[S1 + 1] - Qt[-S1 + 1]) - (Qt[S1 - 1] - Qt[-S1 - 1]));
+            Gs = m2 * (Pt[1] - Pt[-1]) + m1 * (Pt[S1] - Pt[-S1]) +
+                 m3 * ((Pt[S1 + 1] - Pt[-S1 + 1]) - (Pt[S1 - 1] - Pt[-S1 - 1]));
         }
         real w1 = w0, dU = real(0), dV = real(0);
         if (valid) {

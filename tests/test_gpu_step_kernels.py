@@ -1,0 +1,59 @@
+"""The step kernels at the sizes and depths where their variants can go wrong,
+against the FP64 oracle: films around the depth from which Eq. 14's velocity
+factor is 1/h, tile edges and remainders, and non-finite states.
+
+Bars: those of the parity tests, relative L2 1e-10 (FP64) and 1e-4 (FP32) for
+eta, ten times that for P and Q.
+"""
+import numpy as np
+import pytest
+
+from paper_1611_05984_gb300 import scenarios as sc
+from tests.helpers import oracle_from, rel_l2
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL = {"f64": 1e-10, "f32": 1e-4}
+
+
+def _match(s, prec, steps):
+    from paper_1611_05984_gb300 import celeris
+    o = oracle_from(s)
+    g = celeris.from_scenario(s, dtype=torch.float64 if prec == "f64" else torch.float32)
+    o.step(steps)
+    g.step(steps)
+    ref = o.state()
+    got = [a.double().cpu().numpy() for a in g.state()]
+    assert rel_l2(got[0] - s.ws, ref[0] - s.ws) <= TOL[prec]
+    for a, b in zip(got[1:], ref[1:]):
+        if np.linalg.norm(b) > 1e-12:
+            assert rel_l2(a, b) <= 10 * TOL[prec]
+
+
+@pytest.mark.parametrize("friction", [0, 1, 2])
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+def test_films_around_the_desingularisation_depth(prec, friction):
+    """Depths from 0 to three times eps^(1/4) over a bumpy bed, some cells dry
+    and some a film: faces with both, one or no side past the threshold."""
+    rng = np.random.default_rng(3)
+    nx, ny, eps = 70, 45, 1e-4            # threshold depth 0.1 m
+    s = sc.flat_basin(nx, ny, 1.0, 1.0, 0.004, model=1, K=0, friction=friction, fcoef=0.01, eps=eps)
+    s.z = -0.3 + 0.25 * sc.random_bed(nx, ny, 5, 0.0, 1.0, smooth=2)
+    s.w0 = s.z + np.maximum(rng.uniform(-0.05, 0.3, (ny, nx)), 0.0)
+    s.P0 = 0.02 * rng.standard_normal((ny, nx))
+    s.Q0 = 0.02 * rng.standard_normal((ny, nx))
+    _match(s, prec, 3)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("value", [np.nan, -np.nan, np.inf])
+def test_a_non_finite_cell_is_found_after_a_step(prec, value):
+    from paper_1611_05984_gb300 import celeris
+    s = sc.flat_basin(96, 80, 1.0, 2.0, 0.01, K=1)
+    g = celeris.from_scenario(s, dtype=torch.float64 if prec == "f64" else torch.float32)
+    w, P, Q = g.state()
+    P[40, 30] = value
+    g.set_state(w, P, Q)
+    g.step(1)
+    assert not g.check_finite()
