@@ -307,6 +307,7 @@ StencilArgs<real> stencil_args(const cel_solver *s, const Coef<real> &coef, int 
     a.phy = s->phy;
     a.c = coef;
     a.c.gam = s->at<real>(L.gam);
+    make_pairs(a.c, a.kk);
     a.ghost = s->at<real>(L.ghost);
     a.Bc = s->at<real>(L.Bc);
     a.w_in = s->at<real>(L.w[(s->cur + stage) & 1]);
@@ -1344,7 +1345,8 @@ void plan_t(cel_solver *const *ms, int n, EnsPlan &P)
     };
     P.tiles = 0;
     for (int e = 0; e < n; e++)
-        P.tiles += ((ms[e]->geo.nx + kTile - 1) / kTile) * ((ms[e]->geo.ny + kTile - 1) / kTile);
+        P.tiles += ((ms[e]->geo.nx + tile_cols(sizeof(real)) - 1) / tile_cols(sizeof(real))) *
+                   ((ms[e]->geo.ny + tile_rows(sizeof(real)) - 1) / tile_rows(sizeof(real)));
     P.off_tile_desc = take(sizeof(int2) * (size_t)P.tiles);
     // line families grouped by their solver configuration (one launch
     // each), longest lines first within a group
@@ -1936,7 +1938,8 @@ cel_status cel_ensemble_create(cel_solver *const *members, int32_t n, void *tabl
     std::vector<int2> td;
     td.reserve(P.tiles);
     for (int j = 0; j < n; j++) {
-        const int tx = (members[j]->geo.nx + kTile - 1) / kTile, ty = (members[j]->geo.ny + kTile - 1) / kTile;
+        const int cols = tile_cols(e->es), rows = tile_rows(e->es);
+        const int tx = (members[j]->geo.nx + cols - 1) / cols, ty = (members[j]->geo.ny + rows - 1) / rows;
         for (int b = 0; b < tx * ty; b++) td.push_back(make_int2(j, ((b / tx) << 16) | (b % tx)));
     }
     cudaError_t ce = cudaMemcpyAsync(e->tab + e->off_tile_desc, td.data(), sizeof(int2) * td.size(),

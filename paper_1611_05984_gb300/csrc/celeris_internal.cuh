@@ -22,7 +22,7 @@
 
 namespace cel {
 
-constexpr int kTile = 32;          // stencil tile edge (cells)
+constexpr int kTile = 32;          // FP64 stencil tile edge (cells)
 constexpr int kHalo = 2;           // ghost layers (Sec. 2.4)
 constexpr int kTileIn = kTile + 2 * kHalo;   // 36
 constexpr int kStride = kTileIn + 1;         // padded smem row of the state tile
@@ -31,6 +31,11 @@ constexpr int kCornerStride = kCorner + 2;    // odd: a warp reading one corner 
 constexpr int kDcell = kTile + 2;            // 34 cells of d per tile edge
 constexpr int kDStride = kDcell + 1;
 constexpr int kStencilThreads = 256;
+constexpr int kPairCols = 64, kPairWarps = 4;   // FP32 stencil tile: columns (two per lane), warps
+constexpr int kPairRows = 8;                    // its rows per warp where there are tiles enough
+// An ensemble's stencil tiles, per precision.
+inline int tile_cols(int real_bytes) { return real_bytes == 4 ? kPairCols : kTile; }
+inline int tile_rows(int real_bytes) { return real_bytes == 4 ? kPairRows * kPairWarps : kTile; }
 
 enum { kSolid = 0, kSponge = 1, kSine = 2 };
 enum { kBsnq = 0, kNlsw = 1 };
@@ -75,6 +80,7 @@ struct Coef {
     real hwet;           // eps^(1/4): the depth from which Eq. 14's factor is 1/h
     real hgx, hgy;       // g / (2 dx), g / (2 dy) (bed slope from corner sums)
     real Bdg;            // B g
+    real Kx, Ky;         // B g / (2 dx), B g / (2 dy)
     real c6;             // 1 / (24 dx dy) (first-derivative products of F*, G*)
     real B3xy;           // (B + 1/3) / (4 dx dy) (mixed derivatives of F*, G*)
     real ab[3];          // 23, -16, 5 dt / 12 (Eq. 15)
@@ -114,6 +120,8 @@ inline Coef<real> make_coef(const Geo &G, const Phys &p, const Bnd &b)
     c.hgx = real(0.5 * p.g / G.dx);
     c.hgy = real(0.5 * p.g / G.dy);
     c.Bdg = real(p.Bd * p.g);
+    c.Kx = real(p.Bd * p.g * 0.5 / G.dx);
+    c.Ky = real(p.Bd * p.g * 0.5 / G.dy);
     c.c6 = real(1.0 / (24.0 * G.dx * G.dy));
     c.B3xy = real((p.Bd + 1.0 / 3.0) / (4.0 * G.dx * G.dy));
     c.ab[0] = real(23.0 * p.dt / 12.0);
@@ -161,11 +169,33 @@ __device__ __forceinline__ real bbar_at(const real *Bc, const Geo &g, int i, int
                      corner(Bc, g, i + 1, j + 1));
 }
 
+// The FP32 stencil's constants twice over, as its two-cell operations take
+// them (a constant then costs one 64-bit load instead of two moves).
+enum {
+    kcTh2, kcQ, kcMQ, kcHalf, kcTwo, kcMTwo, kcMThree, kcG, kcWs, kcRdx, kcRdy, kcMHgx, kcMHgy, kcMFric, kcRdx2, kcRdy2,
+    kcKx, kcKy, kcC6, kcB3xy, kcDt, kcAb0, kcAb1, kcAb2, kcAm0, kcAm1, kcAm2, kcAm3, kcCount
+};
+template <typename real>
+struct PairConst {};
+template <>
+struct PairConst<float> {
+    float2 v[kcCount];
+};
+inline void make_pairs(const Coef<double> &, PairConst<double> &) {}
+inline void make_pairs(const Coef<float> &c, PairConst<float> &p)
+{
+    const float v[kcCount] = {c.th2, 0.25f, -0.25f, 0.5f, 2.f, -2.f, -3.f, c.g, c.ws, c.rdx, c.rdy, -c.hgx, -c.hgy, -c.fric,
+                              c.rdx2, c.rdy2, c.Kx, c.Ky, c.c6, c.B3xy, c.dt, c.ab[0], c.ab[1], c.ab[2], c.am[0],
+                              c.am[1], c.am[2], c.am[3]};
+    for (int k = 0; k < kcCount; k++) p.v[k] = make_float2(v[k], v[k]);
+}
+
 template <typename real>
 struct StencilArgs {
     Geo geo;
     Phys phy;
     Coef<real> c;
+    PairConst<real> kk;
     const real *ghost;                   // sine-maker ghost table of this step
     const real *Bc;
     const real *w_in, *P_in, *Qc_in;     // state (or AM4 iterate) at time t

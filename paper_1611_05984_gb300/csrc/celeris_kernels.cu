@@ -8,12 +8,14 @@
 //
 // Per step and per stage (predictor, then K corrector iterations) three
 // kernels run:
-//   k_stencil  one 32x32 tile per thread block: stages w, P, Q (+2 ghost
-//              layers produced in shared memory from the boundary rules) and
-//              the bed corners, computes every face flux once, then per cell
-//              E, F, G, F*, G*, friction and the time update; writes w^{n+1},
-//              the increments of U* (row-major) and V* (column-major,
-//              transposed through shared memory) and the dry-cell bits.
+//   k_stencil  one tile per thread block (32x32 in FP64; in FP32
+//              k_stencil_pair, celeris_stencil_f32.cuh): stages w, P, Q (+2
+//              ghost layers produced in shared memory from the boundary
+//              rules) and the bed corners, computes the face fluxes, then per
+//              cell E, F, G, F*, G*, friction and the time update; writes
+//              w^{n+1}, the increments of U* (row-major) and V*
+//              (column-major, transposed through shared memory) and the
+//              dry-cell bits.
 //   k_lines    one thread block per line, x-rows then y-columns: a
 //              partitioned tridiagonal solve of Eq. 21/22 for the increment
 //              P^{n+1} - P^n (each thread eliminates its own segment, the
@@ -21,6 +23,7 @@
 //              reduction), then P^n + increment, sponge and dry-cell epilogue.
 #include "celeris_internal.cuh"
 #include "celeris_physics.cuh"
+#include "celeris_stencil_f32.cuh"
 
 #include <algorithm>
 #include <atomic>
@@ -747,98 +750,8 @@ __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const O
     {
         const int lane = tid & 31, wq = (tid >> 5) & 3;
         const int f0 = wq * 8, f1 = wq == 3 ? kTile + 1 : f0 + 8;
-        if constexpr (sizeof(real) == 8) {
         if (tid < 4 * 32) sweep_faces<real, true>(sm, C, lane, f0, f1);
         else sweep_faces<real, false>(sm, C, lane, f0, f1);
-        } else {
-        const real th = C.theta;
-        real lo[3], hiL[3], hiR[3];
-        // the three cells a reconstruction reads slide along the row (or
-        // column) one cell per face, so each face loads one new cell and one
-        // new pair of corners
-        real wq3[3], Pq[3], Qq[3];
-        if (tid < 4 * 32) {
-            const int r = lane;
-            const int rowo = (r + kHalo) * kStride;
-            const real *cb = sm.Bc + (r + 1) * kCornerStride;
-            real Bf;   // bed at the face about to be computed
-            {
-                const int o = rowo + f0 + 1;
-#pragma unroll
-                for (int u = 0; u < 3; u++) {
-                    wq3[u] = sm.w[o - 1 + u];
-                    Pq[u] = sm.P[o - 1 + u];
-                    Qq[u] = sm.Q[o - 1 + u];
-                }
-                Bf = real(0.5) * (cb[f0 + 1] + cb[f0 + 1 + kCornerStride]);
-                recon(th, wq3, Pq, Qq, real(0.5) * (cb[f0] + cb[f0 + kCornerStride]), Bf, lo, hiL);
-            }
-            for (int f = f0; f < f1; f++) {
-                const int o = rowo + f + 2;           // right cell of face f
-#pragma unroll
-                for (int u = 0; u < 2; u++) {
-                    wq3[u] = wq3[u + 1];
-                    Pq[u] = Pq[u + 1];
-                    Qq[u] = Qq[u + 1];
-                }
-                wq3[2] = sm.w[o + 1];
-                Pq[2] = sm.P[o + 1];
-                Qq[2] = sm.Q[o + 1];
-                const real Bn = real(0.5) * (cb[f + 2] + cb[f + 2 + kCornerStride]);
-                recon(th, wq3, Pq, Qq, Bf, Bn, lo, hiR);
-                real H[3];
-                cu_flux(g, eps, hiL[0], hiL[1], hiL[2], lo[0], lo[1], lo[2], Bf, H);
-                sm.Fx[0][r][f] = H[0];
-                sm.Fx[1][r][f] = H[1];
-                sm.Fx[2][r][f] = H[2];
-                hiL[0] = hiR[0];
-                hiL[1] = hiR[1];
-                hiL[2] = hiR[2];
-                Bf = Bn;
-            }
-        } else {
-            const int c = lane;
-            const int tx = c + kHalo;
-            const real *cb = sm.Bc + c + 1;
-            real Bf;
-            {
-                const int o = (f0 + 1) * kStride + tx;
-#pragma unroll
-                for (int u = 0; u < 3; u++) {
-                    wq3[u] = sm.w[o + (u - 1) * kStride];
-                    Pq[u] = sm.P[o + (u - 1) * kStride];
-                    Qq[u] = sm.Q[o + (u - 1) * kStride];
-                }
-                Bf = real(0.5) * (cb[(f0 + 1) * kCornerStride] + cb[(f0 + 1) * kCornerStride + 1]);
-                recon(th, wq3, Pq, Qq, real(0.5) * (cb[f0 * kCornerStride] + cb[f0 * kCornerStride + 1]), Bf, lo,
-                      hiL);
-            }
-            for (int gq = f0; gq < f1; gq++) {
-                const int o = (gq + 2) * kStride + tx;  // north cell of face gq
-#pragma unroll
-                for (int u = 0; u < 2; u++) {
-                    wq3[u] = wq3[u + 1];
-                    Pq[u] = Pq[u + 1];
-                    Qq[u] = Qq[u + 1];
-                }
-                wq3[2] = sm.w[o + kStride];
-                Pq[2] = sm.P[o + kStride];
-                Qq[2] = sm.Q[o + kStride];
-                const real Bn = real(0.5) * (cb[(gq + 2) * kCornerStride] + cb[(gq + 2) * kCornerStride + 1]);
-                recon(th, wq3, Pq, Qq, Bf, Bn, lo, hiR);
-                real H[3];
-                // normal discharge is Q, tangential is P
-                cu_flux(g, eps, hiL[0], hiL[2], hiL[1], lo[0], lo[2], lo[1], Bf, H);
-                sm.Fy[0][gq][c] = H[0];
-                sm.Fy[1][gq][c] = H[2];
-                sm.Fy[2][gq][c] = H[1];
-                hiL[0] = hiR[0];
-                hiL[1] = hiR[1];
-                hiL[2] = hiR[2];
-                Bf = Bn;
-            }
-        }
-        }
     }
     __syncthreads();
 
@@ -945,12 +858,34 @@ __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const O
     if (tid < kTile && O.x0() + tid < nx) A.mask_c[(size_t)(O.x0() + tid) * G.nwy + (O.y0() >> 5)] = sm.colbits[tid];
 }
 
-template <typename real, int kSpec>
-__global__ void __launch_bounds__(kStencilThreads, sizeof(real) == 4 ? 4 : 2) k_stencil(const __grid_constant__ StencilArgs<real> A)
+template <int kSpec>
+__global__ void __launch_bounds__(kStencilThreads, 2) k_stencil(const __grid_constant__ StencilArgs<double> A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     dependent_launch_wait_then_release();
-    stencil_tile<real, kSpec>(A, GridOrigin(), smem_raw);
+    stencil_tile<double, kSpec>(A, GridOrigin(), smem_raw);
+}
+
+// FP32 (celeris_stencil_f32.cuh): 64 columns and 4 kR rows per block.
+struct BlockBarrier {
+    __device__ __forceinline__ void operator()() const { __syncthreads(); }
+};
+// The barrier of one half of a 256-thread block.
+struct HalfBarrier {
+    int id;
+    __device__ __forceinline__ void operator()() const
+    {
+        asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kPThreads) : "memory");
+    }
+};
+
+template <int kSpec, int kR>
+__global__ void __launch_bounds__(kPThreads, 4) k_stencil_pair(const __grid_constant__ StencilArgs<float> A)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    dependent_launch_wait_then_release();
+    stencil_tile_pair<kSpec, kR>(A, blockIdx.x * kPW, blockIdx.y * PairSmem<kR>::TH, smem_raw, threadIdx.x,
+                                 BlockBarrier());
 }
 
 // Copy a scenario's argument block (device memory) into shared memory.
@@ -966,12 +901,12 @@ __device__ __forceinline__ void load_args(T &dst, const T *src)
 // Ensemble: the tiles of every member in one launch.  desc[b] names block
 // b's member (x) and tile (y: row << 16 | column); the member's arguments
 // are copied to shared memory.
-template <typename real, int kSpec>
-__global__ void __launch_bounds__(kStencilThreads, sizeof(real) == 4 ? 4 : 2)
-    k_stencil_batch(const StencilArgs<real> *__restrict__ args, const int2 *__restrict__ desc)
+template <int kSpec>
+__global__ void __launch_bounds__(kStencilThreads, 2)
+    k_stencil_batch(const StencilArgs<double> *__restrict__ args, const int2 *__restrict__ desc)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ __align__(16) StencilArgs<real> A;
+    __shared__ __align__(16) StencilArgs<double> A;
     __shared__ int origin[2];
     const int2 d = desc[blockIdx.x];
     if (threadIdx.x == 0) {
@@ -980,7 +915,20 @@ __global__ void __launch_bounds__(kStencilThreads, sizeof(real) == 4 ? 4 : 2)
     }
     load_args(A, args + d.x);
     __syncthreads();
-    stencil_tile<real, kSpec>(A, SharedOrigin{origin}, smem_raw);
+    stencil_tile<double, kSpec>(A, SharedOrigin{origin}, smem_raw);
+}
+
+template <int kSpec>
+__global__ void __launch_bounds__(kPThreads, 4)
+    k_stencil_pair_batch(const StencilArgs<float> *__restrict__ args, const int2 *__restrict__ desc)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ __align__(16) StencilArgs<float> A;
+    const int2 d = desc[blockIdx.x];
+    load_args(A, args + d.x);
+    __syncthreads();
+    stencil_tile_pair<kSpec, kPairRows>(A, (d.y & 0xffff) * kPW, (d.y >> 16) * PairSmem<kPairRows>::TH, smem_raw,
+                                        threadIdx.x, BlockBarrier());
 }
 
 // ------------------------------------------------------------ line solves
@@ -997,23 +945,6 @@ __device__ __forceinline__ void coef23(real B3, real hrh, real srh, real rh2, re
     b = real(1) + real(2) * r;
     c = -s - r;
 }
-
-// Asynchronous copy of one element from global to shared memory (zero-filled
-// when !valid, reading nothing); all of a thread's copies are in flight at
-// once and cost no registers.  cp_async_wait_all waits for this thread's.
-template <typename real>
-__device__ __forceinline__ void cp_async_elem(real *smem, const real *gmem, bool valid)
-{
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    if (sizeof(real) == 4)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(s), "l"(gmem), "r"(valid ? 4 : 0)
-                     : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(s), "l"(gmem), "r"(valid ? 8 : 0)
-                     : "memory");
-}
-
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Shared-memory slot of line element k: element j of segment t sits at
 // j * sp + t (sp odd), so the threads of a warp sweeping their segments touch
@@ -1863,12 +1794,22 @@ __device__ __noinline__ bool grid_sync(unsigned *bar, unsigned expect, long long
 // The arguments sit in shared memory and nothing the work stores aliases
 // them, which the compiler is told so that it keeps them in registers
 // across the global stores.
-template <typename real, int kSpec>
-__device__ __noinline__ void persist_tile(const StencilArgs<real> &__restrict__ A, const int *origin,
+template <int kSpec>
+__device__ __noinline__ void persist_tile(const StencilArgs<double> &__restrict__ A, const int *origin,
                                           unsigned char *smem_raw)
 {
     __builtin_assume(__isShared(&A));
-    stencil_tile<real, kSpec>(A, SharedOrigin{origin}, smem_raw);
+    stencil_tile<double, kSpec>(A, SharedOrigin{origin}, smem_raw);
+}
+
+// FP32: each half of the block takes a tile of its own (kPThreads threads).
+template <int kSpec>
+__device__ __noinline__ void persist_tile(const StencilArgs<float> &__restrict__ A, const int *origin,
+                                          unsigned char *smem_raw)
+{
+    __builtin_assume(__isShared(&A));
+    stencil_tile_pair<kSpec, kPairRows>(A, origin[0], origin[1], smem_raw, threadIdx.x & (kPThreads - 1),
+                                        HalfBarrier{1 + (int)threadIdx.x / kPThreads});
 }
 
 template <typename real, int M>
@@ -1892,17 +1833,26 @@ __device__ __forceinline__ void persist_flag(unsigned *bar, unsigned code, unsig
 // batched launch would end.  Every block runs the same loop, so each takes
 // every barrier.
 template <typename real>
-__global__ void __launch_bounds__(kStencilThreads, sizeof(real) == 4 ? 4 : 2)
+__host__ __device__ constexpr size_t persist_smem()
+{
+    return sizeof(real) == 4 ? (kStencilThreads / kPThreads) * sizeof(PairSmem<kPairRows>) : sizeof(StencilSmem<double>);
+}
+
+template <typename real>
+__global__ void __launch_bounds__(kStencilThreads, 2)
     k_ensemble_persistent(const __grid_constant__ PersistArgs<real> P)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ __align__(16) StencilArgs<real> As;
-    __shared__ int origin[2];
+    // tiles side by side in the block, and threads of each
+    constexpr int kSide = sizeof(real) == 4 ? kStencilThreads / kPThreads : 1, kOwn = kStencilThreads / kSide;
+    constexpr int kTX = sizeof(real) == 4 ? kPW : kTile, kTY = sizeof(real) == 4 ? PairSmem<kPairRows>::TH : kTile;
+    static_assert(sizeof(PairSmem<kPairRows>) % 16 == 0, "tiles side by side keep their alignment");
+    __shared__ __align__(16) StencilArgs<real> As[kSide];
+    __shared__ int origin[kSide][2];
     __shared__ int item;
     // the line phases reuse the stencil's shared memory: a slot's arguments,
     // then the values that cross warps
-    static_assert(sizeof(LineArgs<real>) * (kStencilThreads / 32) + sizeof(LineShared<real>) <=
-                      sizeof(StencilSmem<real>),
+    static_assert(sizeof(LineArgs<real>) * (kStencilThreads / 32) + sizeof(LineShared<real>) <= persist_smem<real>(),
                   "line phase shared memory");
     LineArgs<real> *Al = reinterpret_cast<LineArgs<real> *>(smem_raw);
     LineShared<real> &L =
@@ -1946,28 +1896,40 @@ __global__ void __launch_bounds__(kStencilThreads, sizeof(real) == 4 ? 4 : 2)
             const unsigned char *ent = P.entries + (size_t)ei * P.entry_bytes;
             const StencilArgs<real> *sa = reinterpret_cast<const StencilArgs<real> *>(ent);
             const int spec = P.spec[stage];
-            for (int t = next_item(); t < P.tiles; t = next_item()) {
-                const int2 d = P.tile_desc[t];
-                if (d.x < 0 || d.x >= P.nmembers) {
-                    if (threadIdx.x == 0) persist_flag(P.bar, 1u, (unsigned)t);
-                    continue;
+            for (int p = next_item(); p * kSide < P.tiles; p = next_item()) {
+                const int half = threadIdx.x / kOwn, t = p * kSide + half, own = threadIdx.x - half * kOwn;
+                int2 d = make_int2(-1, 0);
+                bool ok = t < P.tiles;
+                if (ok) {
+                    d = P.tile_desc[t];
+                    if (d.x < 0 || d.x >= P.nmembers) {
+                        if (own == 0) persist_flag(P.bar, 1u, (unsigned)t);
+                        ok = false;
+                    }
                 }
-                if (threadIdx.x == 0) {
-                    origin[0] = (d.y & 0xffff) * kTile;
-                    origin[1] = (d.y >> 16) * kTile;
+                if (ok) {
+                    if (own == 0) {
+                        origin[half][0] = (d.y & 0xffff) * kTX;
+                        origin[half][1] = (d.y >> 16) * kTY;
+                    }
+                    const int nw = (int)(sizeof(StencilArgs<real>) / sizeof(int));
+                    int *dst = reinterpret_cast<int *>(&As[half]);
+                    const int *src = reinterpret_cast<const int *>(sa + d.x);
+                    for (int k = own; k < nw; k += kOwn) dst[k] = src[k];
                 }
-                load_args(As, sa + d.x);
                 __syncthreads();
-                if ((d.y & 0xffff) * kTile >= As.geo.nx || (d.y >> 16) * kTile >= As.geo.ny) {
-                    if (threadIdx.x == 0) persist_flag(P.bar, 2u, (unsigned)t);
-                    continue;
+                if (ok && ((d.y & 0xffff) * kTX >= As[half].geo.nx || (d.y >> 16) * kTY >= As[half].geo.ny)) {
+                    if (own == 0) persist_flag(P.bar, 2u, (unsigned)t);
+                    ok = false;
                 }
+                if (!ok) continue;   // this tile's threads wait at the next item
+                unsigned char *sm = smem_raw + (sizeof(real) == 4 ? half * sizeof(PairSmem<kPairRows>) : 0);
                 if (spec == 1)
-                    persist_tile<real, 1>(As, origin, smem_raw);
+                    persist_tile<1>(As[half], origin[half], sm);
                 else if (spec == 2)
-                    persist_tile<real, 2>(As, origin, smem_raw);
+                    persist_tile<2>(As[half], origin[half], sm);
                 else
-                    persist_tile<real, 0>(As, origin, smem_raw);
+                    persist_tile<0>(As[half], origin[half], sm);
             }
             if (!end_phase()) return;
             const LineArgs<real> *la = reinterpret_cast<const LineArgs<real> *>(ent + P.sarg_bytes);
@@ -2163,13 +2125,13 @@ cudaError_t launch_ghost_table(const Geo &g, const Phys &p, const Bnd &b, const 
     return cudaGetLastError();
 }
 
-template <typename real>
-cudaError_t launch_stencil(const StencilArgs<real> &a, cudaStream_t st)
+template <>
+cudaError_t launch_stencil<double>(const StencilArgs<double> &a, cudaStream_t st)
 {
     static bool configured[3] = {false, false, false};
-    const size_t smem = sizeof(StencilSmem<real>);
+    const size_t smem = sizeof(StencilSmem<double>);
     const int spec = stencil_spec(a);
-    auto *kern = spec == 1 ? k_stencil<real, 1> : spec == 2 ? k_stencil<real, 2> : k_stencil<real, 0>;
+    auto *kern = spec == 1 ? k_stencil<1> : spec == 2 ? k_stencil<2> : k_stencil<0>;
     if (!configured[spec]) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -2179,6 +2141,42 @@ cudaError_t launch_stencil(const StencilArgs<real> &a, cudaStream_t st)
     cudaError_t e = launch_step_kernel(kern, grid, dim3(kStencilThreads), smem, st, a);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
+}
+
+namespace {
+
+template <int kR>
+cudaError_t launch_stencil_pair(const StencilArgs<float> &a, cudaStream_t st)
+{
+    static bool configured[3] = {false, false, false};
+    constexpr size_t smem = sizeof(PairSmem<kR>);
+    const int spec = stencil_spec(a);
+    auto *kern = spec == 1 ? k_stencil_pair<1, kR> : spec == 2 ? k_stencil_pair<2, kR> : k_stencil_pair<0, kR>;
+    if (!configured[spec]) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        configured[spec] = true;
+    }
+    dim3 grid((a.geo.nx + kPW - 1) / kPW, (a.geo.ny + PairSmem<kR>::TH - 1) / PairSmem<kR>::TH);
+    cudaError_t e = launch_step_kernel(kern, grid, dim3(kPThreads), smem, st, a);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+}  // namespace
+
+template <>
+cudaError_t launch_stencil<float>(const StencilArgs<float> &a, cudaStream_t st)
+{
+    // Rows per warp, by the number of 64 x 32 tiles (608 blocks fit the GPU at
+    // once): 8 need the fewest instructions per cell, and win once there are
+    // enough tiles to keep the SMs evenly loaded; fewer rows give more and
+    // shorter blocks.  Step in us with 8 / 4 / 2 rows: 2048 x 2048 (2048
+    // tiles) 272 / - / 277; 1024 x 1024 (512) 89 / 84 / 86; 601 x 601 (190)
+    // 55 / 46 / 46; 512 x 512 (128) 47 / 37 / 37; 256 x 256 (32) 46 / 32 / 26.
+    const long tiles = (long)((a.geo.nx + kPW - 1) / kPW) * ((a.geo.ny + 31) / 32);
+    if (tiles >= 1024) return launch_stencil_pair<kPairRows>(a, st);
+    if (tiles >= 152) return launch_stencil_pair<4>(a, st);
+    return launch_stencil_pair<2>(a, st);
 }
 
 // The ensemble's batched launches are plain launches: replayed as captured
@@ -2207,14 +2205,24 @@ cudaError_t launch_stencil_batch(const StencilArgs<real> *args, const int2 *desc
 {
     static bool configured[3] = {false, false, false};
     if (spec < 0 || spec > 2) return cudaErrorInvalidValue;
-    const size_t smem = sizeof(StencilSmem<real>);
-    auto *kern = spec == 1 ? k_stencil_batch<real, 1> : spec == 2 ? k_stencil_batch<real, 2> : k_stencil_batch<real, 0>;
+    void (*kern)(const StencilArgs<real> *, const int2 *);
+    size_t smem;
+    int threads;
+    if constexpr (sizeof(real) == 4) {
+        kern = spec == 1 ? k_stencil_pair_batch<1> : spec == 2 ? k_stencil_pair_batch<2> : k_stencil_pair_batch<0>;
+        smem = sizeof(PairSmem<kPairRows>);
+        threads = kPThreads;
+    } else {
+        kern = spec == 1 ? k_stencil_batch<1> : spec == 2 ? k_stencil_batch<2> : k_stencil_batch<0>;
+        smem = sizeof(StencilSmem<double>);
+        threads = kStencilThreads;
+    }
     if (!configured[spec]) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         configured[spec] = true;
     }
-    if (nblocks > 0) kern<<<nblocks, kStencilThreads, smem, st>>>(args, desc);
+    if (nblocks > 0) kern<<<nblocks, threads, smem, st>>>(args, desc);
     return cudaGetLastError();
 }
 
@@ -2464,7 +2472,7 @@ int persistent_grid()
     std::call_once(init, [] {
         for (auto &g : grid) g.store(-1);
     });
-    const size_t smem = sizeof(StencilSmem<real>);
+    const size_t smem = persist_smem<real>();
     int dev = 0, sms = 0, per = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) {
         cudaGetLastError();
@@ -2488,7 +2496,7 @@ template <typename real>
 cudaError_t launch_persistent(const PersistArgs<real> &p, int grid, cudaStream_t st)
 {
     if (grid <= 0 || p.nstages > kPersistMaxStages || p.nruns > kPersistMaxRuns) return cudaErrorInvalidValue;
-    const size_t smem = sizeof(StencilSmem<real>);
+    const size_t smem = persist_smem<real>();
     void *params[] = {const_cast<PersistArgs<real> *>(&p)};
     return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_ensemble_persistent<real>), dim3(grid),
                                        dim3(kStencilThreads), params, smem, st);
@@ -2527,7 +2535,6 @@ cudaError_t launch_persistent(const PersistArgs<real> &p, int grid, cudaStream_t
     template cudaError_t launch_ghost_table<real>(const Geo &, const Phys &, const Bnd &, const real *,   \
                                                   const double *, double, double, real *, int,          \
                                                   cudaStream_t);                                        \
-    template cudaError_t launch_stencil<real>(const StencilArgs<real> &, cudaStream_t);                  \
     template cudaError_t launch_lines<real>(const LinePair<real> &, cudaStream_t);                       \
     template cudaError_t launch_lines_transposed<real>(const LinePair<real> &, cudaStream_t);            \
     template cudaError_t launch_lines_solution<real>(const LinePair<real> &, cudaStream_t);              \

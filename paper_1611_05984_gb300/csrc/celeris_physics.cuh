@@ -208,7 +208,7 @@ __device__ __forceinline__ float minmod_r(float a, float b, float c)
     float lo, hi;
     asm("min.ftz.f32 %0, %1, %2, %3;" : "=f"(lo) : "f"(a), "f"(b), "f"(c));
     asm("max.ftz.f32 %0, %1, %2, %3;" : "=f"(hi) : "f"(a), "f"(b), "f"(c));
-    return fmaxf(lo, 0.f) + fminf(hi, 0.f);
+    return fmaxf(lo, fminf(hi, 0.f));   // 0 clamped to [lo, hi]
 }
 __device__ __forceinline__ double minmod_r(double a, double b, double c)
 {

@@ -57,3 +57,36 @@ def test_a_non_finite_cell_is_found_after_a_step(prec, value):
     g.set_state(w, P, Q)
     g.step(1)
     assert not g.check_finite()
+
+
+# The FP32 stencil's tiles are 64 columns by 32, 16 or 8 rows (by the number of
+# tiles), the FP64 stencil's 32 columns: one column or row short of, at and past
+# their edges, odd widths (a lane's second cell outside), and each height.
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("nx,ny", [(2, 2), (63, 7), (64, 8), (65, 9), (66, 33), (127, 31), (129, 32), (191, 65),
+                                   (705, 450), (1345, 1500)])
+def test_tile_edges_and_remainders(prec, nx, ny):
+    """Waves towards a beach, with a maker on the west, sponges and a dry
+    shore, over the Euler start-up and full steps."""
+    if prec == "f64" and nx * ny > 500000:
+        pytest.skip("the tall FP32 tiles' size")
+    dx = max(1.0, 430.0 / nx)
+    s = sc.beach(nx=nx, ny=ny, dx=dx, sponge=max(1, min(50, ny // 8)))
+    x = (np.arange(nx) + 0.5) * dx
+    y = (np.arange(ny) + 0.5) * dx
+    s.w0 = np.maximum(s.z, 0.2 * np.sin(0.09 * x)[None, :] * np.cos(0.05 * y)[:, None])
+    s.P0 = 0.5 * np.where(s.z < -0.5, s.w0, 0.0)
+    s.Q0 = 0.2 * np.where(s.z < -0.5, s.w0, 0.0)
+    _match(s, prec, 5)
+
+
+@pytest.mark.parametrize("K,model", [(0, 0), (2, 0), (1, 1)])
+def test_carries_correctors_and_shallow_water_across_tiles(K, model):
+    """The predictor-only carries, two corrector stages and the shallow-water
+    model on a grid of several FP32 tiles with makers on all sides."""
+    s = sc.flat_basin(150, 70, 1.0, 1.0, 0.02, model=model, K=K, friction=1, fcoef=0.01, eps=1e-8)
+    s.z = -1.0 + 0.3 * sc.random_bed(150, 70, 6, -1.0, 1.0, smooth=4)
+    for side in (sc.W, sc.E, sc.S, sc.N):
+        s.sides[side] = sc.Side(sc.SINE, 0, ((0.02, 3.0, 0.3 + side, 0.1 * side),))
+    for prec in ("f32", "f64"):
+        _match(s, prec, 6)
