@@ -946,6 +946,16 @@ __device__ __forceinline__ void coef23(real B3, real hrh, real srh, real rh2, re
     c = -s - r;
 }
 
+// The same from the constants folded per line (register path).
+template <typename real>
+__device__ __forceinline__ void coef23_folded(real kr, real ks, real dd, real dm, real dp, real &a, real &b, real &c)
+{
+    const real r = (dd * dd) * kr, s = (dd * ks) * (dp - dm);
+    a = s - r;
+    b = real(1) + real(2) * r;
+    c = -s - r;
+}
+
 // Shared-memory slot of line element k: element j of segment t sits at
 // j * sp + t (sp odd), so the threads of a warp sweeping their segments touch
 // consecutive words at every step (no bank conflicts).
@@ -974,14 +984,16 @@ constexpr unsigned kFull = 0xffffffffu;
 // Cyclic reduction of a warp's 32 rows a x_{i-1} + b x_i + c x_{i+1} = r
 // (rows beyond the warp decoupled), NR right sides at once: afterwards row i
 // reads b x_i = r.  Where only the first `rows` rows couple (the rest are
-// identity rows), ceil(log2(rows)) levels decouple them.
+// identity rows), ceil(log2(rows)) levels decouple them.  a of the first and
+// c of the last coupled row are 0, so the shuffles' own values at the warp's
+// ends are multiplied by 0.
 template <typename real, int NR>
-__device__ __forceinline__ void warp_cr(real &a, real &b, real &c, real (&r)[NR], int lane, int rows = 32)
+__device__ __forceinline__ void warp_cr(real &a, real &b, real &c, real (&r)[NR], int rows = 32)
 {
 #pragma unroll
     for (int s = 1; s < 32; s <<= 1) {
         if (s >= rows) break;
-        const real ib = real(1) / b;   // each row's reciprocal, once, to both neighbours
+        const real ib = rcp_r(b);   // each row's reciprocal, once, to both neighbours
         const real am = __shfl_up_sync(kFull, a, s), ibm = __shfl_up_sync(kFull, ib, s);
         const real cm = __shfl_up_sync(kFull, c, s);
         const real ap = __shfl_down_sync(kFull, a, s), ibp = __shfl_down_sync(kFull, ib, s);
@@ -992,8 +1004,7 @@ __device__ __forceinline__ void warp_cr(real &a, real &b, real &c, real (&r)[NR]
             rm[q] = __shfl_up_sync(kFull, r[q], s);
             rp[q] = __shfl_down_sync(kFull, r[q], s);
         }
-        const real k1 = lane >= s ? a * ibm : real(0);
-        const real k2 = lane + s < 32 ? c * ibp : real(0);
+        const real k1 = a * ibm, k2 = c * ibp;
         b = b - cm * k1 - ap * k2;
 #pragma unroll
         for (int q = 0; q < NR; q++) r[q] = r[q] - rm[q] * k1 - rp[q] * k2;
@@ -1072,7 +1083,7 @@ __device__ __forceinline__ void t_row(const LineArgs<real> &A, int k, real dm, r
         b = real(1);
         return;
     }
-    coef23(A.c.B3, A.hrh, A.srh, A.rh2, dd, dm, dp, a, b, c);
+    coef23_folded(A.kr, A.ks, dd, dm, dp, a, b, c);
     if (k == 0) {
         if (!lo_sine) b -= a;
         else if (rk) *rk -= a * lo_inc;
@@ -1123,6 +1134,7 @@ __device__ __forceinline__ void line_solve_reg(const LineArgs<real> &A, int line
     const size_t lo = (size_t)line * A.pitch;
     real *out = A.sol + lo;
     const bool any = act && f < n;         // the segment holds rows of the line
+    const bool full = f + M <= n;          // and no others
 
     // What the kernel before this one on the stream does not write comes
     // first: P^n (read in the epilogue: to L1 now), the depths, the rows of
@@ -1140,9 +1152,11 @@ __device__ __forceinline__ void line_solve_reg(const LineArgs<real> &A, int line
             if (kMode == 0)   // the dry bits, read in the epilogue
                 asm volatile("prefetch.global.L1 [%0];" ::"l"(A.mask + (size_t)line * A.nwords + (f >> 5)));
             load_run<real, M>(r, A.rhs + lo + f);
+            if (!full) {
 #pragma unroll
-            for (int j = 0; j < M; j++)
-                if (f + j >= n) r[j] = real(0);
+                for (int j = 0; j < M; j++)
+                    if (f + j >= n) r[j] = real(0);
+            }
         } else {
 #pragma unroll
             for (int j = 0; j < M; j++) r[j] = real(0);
@@ -1161,7 +1175,13 @@ __device__ __forceinline__ void line_solve_reg(const LineArgs<real> &A, int line
             real mid[M];
             load_run<real, M>(mid, dl + f);
 #pragma unroll
-            for (int j = 0; j < M; j++) dv[j + 2] = f + j < n ? mid[j] : dl[n - 1];
+            for (int j = 0; j < M; j++) dv[j + 2] = mid[j];
+            if (!full) {
+                const real last = dl[n - 1];
+#pragma unroll
+                for (int j = 0; j < M; j++)
+                    if (f + j >= n) dv[j + 2] = last;
+            }
             dv[0] = dl[f >= 2 ? f - 2 : 0];
             dv[1] = dl[f >= 1 ? f - 1 : 0];
             dv[M + 2] = dl[f + M < n ? f + M : n - 1];
@@ -1179,7 +1199,7 @@ __device__ __forceinline__ void line_solve_reg(const LineArgs<real> &A, int line
             real ta[M + 2], tb[M + 2], tc[M + 2];   // T's rows f - 1 .. f + M
 #pragma unroll
             for (int j = 0; j < M + 2; j++)
-                coef23(A.c.B3, A.hrh, A.srh, A.rh2, dv[j + 1], dv[j], dv[j + 2], ta[j], tb[j], tc[j]);
+                coef23_folded(A.kr, A.ks, dv[j + 1], dv[j], dv[j + 2], ta[j], tb[j], tc[j]);
             if (f == 0 || at_end) {
 #pragma unroll
                 for (int j = 0; j < M + 2; j++)
@@ -1196,7 +1216,7 @@ __device__ __forceinline__ void line_solve_reg(const LineArgs<real> &A, int line
         } else {
 #pragma unroll
             for (int j = 0; j < M; j++)
-                coef23(A.c.B3, A.hrh, A.srh, A.rh2, dv[j + 2], dv[j + 1], dv[j + 3], ra[j], rb[j], rc[j]);
+                coef23_folded(A.kr, A.ks, dv[j + 2], dv[j + 1], dv[j + 3], ra[j], rb[j], rc[j]);
             // the makers' ghost increments (t^{n+1} - t^n) at the line's ends
             // and the coefficients that carry them to the right side
             real lo_inc = real(0), hi_inc = real(0), a_lo = real(0), c_hi = real(0);
@@ -1226,32 +1246,38 @@ __device__ __forceinline__ void line_solve_reg(const LineArgs<real> &A, int line
                     if (f + j == n - 1) r[j] -= c_hi * hi_inc;
             }
         }
-        // Thomas on rows f .. f + M - 2 against (r, -a_f e_0, -c e_last)
-        real g[m1], y[m1], uu[m1], vv[m1];
+        // Thomas on rows f .. f + M - 2 against (r, -a_f e_0, -c e_last): the
+        // rows' own factors and the couplings' columns first, which need no
+        // right side, so that its load is in flight meanwhile; ra becomes
+        // a / pivot, rb 1 / pivot and rc c / pivot
+        real y[m1], uu[m1], vv[m1];
         real Y = real(0), U = real(0), V = real(0);
-        {
-            real gp = real(0), yp = real(0), up = real(0);
+        const real al = ra[m1], bl = rb[m1], cl = rc[m1];
+        rb[0] = rcp_r(rb[0]);
+        ra[0] *= rb[0];
+        rc[0] *= rb[0];
+        uu[0] = -ra[0];
 #pragma unroll
-            for (int j = 0; j < m1; j++) {
-                const real inv = real(1) / (rb[j] - ra[j] * gp);
-                g[j] = j + 1 < m1 ? rc[j] * inv : real(0);
-                y[j] = (r[j] - ra[j] * yp) * inv;
-                uu[j] = (j == 0 ? -ra[0] : -ra[j] * up) * inv;
-                vv[j] = j + 1 == m1 ? -rc[j] * inv : real(0);
-                gp = g[j];
-                yp = y[j];
-                up = uu[j];
-            }
-#pragma unroll
-            for (int j = m1 - 2; j >= 0; j--) {
-                y[j] -= g[j] * y[j + 1];
-                uu[j] -= g[j] * uu[j + 1];
-                vv[j] = -g[j] * vv[j + 1];
-            }
+        for (int j = 1; j < m1; j++) {
+            rb[j] = rcp_r(rb[j] - ra[j] * rc[j - 1]);
+            ra[j] *= rb[j];
+            rc[j] *= rb[j];
+            uu[j] = -ra[j] * uu[j - 1];
         }
+        vv[m1 - 1] = -rc[m1 - 1];
+#pragma unroll
+        for (int j = m1 - 2; j >= 0; j--) {
+            uu[j] -= rc[j] * uu[j + 1];
+            vv[j] = -rc[j] * vv[j + 1];
+        }
+        y[0] = r[0] * rb[0];
+#pragma unroll
+        for (int j = 1; j < m1; j++) y[j] = r[j] * rb[j] - ra[j] * y[j - 1];
+#pragma unroll
+        for (int j = m1 - 2; j >= 0; j--) y[j] -= rc[j] * y[j + 1];
         // the separator's row in (s_{t-1}, s_t, s_{t+1}): the next thread's
         // first interior row by shuffle (lane 31: later, from shared memory)
-        const real al = ra[m1], bl = rb[m1], cl = rc[m1], rl = r[m1];
+        const real rl = r[m1];
         if (act) {
         const real ny0 = __shfl_down_sync(kFull, y[0], 1), nu0 = __shfl_down_sync(kFull, uu[0], 1);
         const real nv0 = __shfl_down_sync(kFull, vv[0], 1);
@@ -1275,8 +1301,8 @@ __device__ __forceinline__ void line_solve_reg(const LineArgs<real> &A, int line
             b1 = real(1);
             rr1[0] = real(0);
         }
-        warp_cr<real, 3>(a1, b1, c1, rr1, lane);
-        const real ib = real(1) / b1;
+        warp_cr<real, 3>(a1, b1, c1, rr1);
+        const real ib = rcp_r(b1);
         Y = rr1[0] * ib;
         U = rr1[1] * ib;
         V = rr1[2] * ib;
@@ -1322,8 +1348,8 @@ __device__ __forceinline__ void line_solve_reg(const LineArgs<real> &A, int line
                 C2 = C1 * q2;
                 R2[0] = R1 - A1 * sh30[lane][0] - C1 * q0;
             }
-            warp_cr<real, 1>(A2, B2, C2, R2, lane, nw);
-            if (lane < nw) shS[lane] = R2[0] / B2;
+            warp_cr<real, 1>(A2, B2, C2, R2, nw);
+            if (lane < nw) shS[lane] = R2[0] * rcp_r(B2);
         }
         __syncthreads();
         if (!act) return;
