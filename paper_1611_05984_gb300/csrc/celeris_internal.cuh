@@ -79,7 +79,6 @@ struct Coef {
     real th2;            // 2 theta (slopes before their factor 1/4)
     real hwet;           // eps^(1/4): the depth from which Eq. 14's factor is 1/h
     real hgx, hgy;       // g / (2 dx), g / (2 dy) (bed slope from corner sums)
-    real Bdg;            // B g
     real Kx, Ky;         // B g / (2 dx), B g / (2 dy)
     real c6;             // 1 / (24 dx dy) (first-derivative products of F*, G*)
     real B3xy;           // (B + 1/3) / (4 dx dy) (mixed derivatives of F*, G*)
@@ -119,7 +118,6 @@ inline Coef<real> make_coef(const Geo &G, const Phys &p, const Bnd &b)
     c.hwet = real(std::sqrt(std::sqrt(p.eps)));
     c.hgx = real(0.5 * p.g / G.dx);
     c.hgy = real(0.5 * p.g / G.dy);
-    c.Bdg = real(p.Bd * p.g);
     c.Kx = real(p.Bd * p.g * 0.5 / G.dx);
     c.Ky = real(p.Bd * p.g * 0.5 / G.dy);
     c.c6 = real(1.0 / (24.0 * G.dx * G.dy));

@@ -389,16 +389,17 @@ __global__ void k_ghost_batch(const GhostArgs<real> *__restrict__ args, const in
 
 // ------------------------------------------------------------ the stencil
 
-template <typename real>
+// A tile of 32 columns and TY rows.
+template <typename real, int TY>
 struct StencilSmem {
-    real w[kTileIn * kStride];
-    real P[kTileIn * kStride];
-    real Q[kTileIn * kStride];
-    real Bc[kCorner * kCornerStride];
-    real d[kDcell * kDStride];
-    real Fx[3][kTile][kTile + 1];    // x-faces: [component][row][face]
-    real Fy[3][kTile + 1][kTile];    // y-faces: [component][face][column]
-    real Vout[kTile][kTile + 1];     // V*^{n+1} staged for the transposed store
+    real w[(TY + 4) * kStride];
+    real P[(TY + 4) * kStride];
+    real Q[(TY + 4) * kStride];
+    real Bc[(TY + 3) * kCornerStride];
+    real d[(TY + 2) * kDStride];
+    real Fx[3][TY][kTile + 1];    // x-faces: [component][row][face]
+    real Fy[3][TY + 1][kTile];    // y-faces: [component][face][column]
+    real Vout[TY][kTile + 1];     // V*^{n+1} staged for the transposed store
     uint32_t colbits[kTile];
 };
 
@@ -479,18 +480,27 @@ __device__ __forceinline__ real advance(const StencilArgs<real> &A, int v, real 
     const int kind = stage_kind<kSpec>(A);
     const bool ring = stage_ring<kSpec>(A);
     const Coef<real> &C = A.c;
-    if (kind == kAM4) return c.Y + C.am[0] * R + Phi;
+    if (kind == kAM4) {
+        const real s = fma(C.am[0], R, c.Y);
+        return v > 0 ? add_r(s, Phi) : s;
+    }
     if (ring) {
         real D;
         if (kind == kEuler0) {
-            D = C.dt * R;
+            D = mul_r(C.dt, R);
         } else if (kind == kEuler1) {
-            D = C.dt * R + (Phi - c.p1);
+            D = mul_r(C.dt, R);
+            if (v > 0) D = add_r(D, sub_r(Phi, c.p1));
         } else {
-            D = C.ab[0] * R + C.ab[1] * c.r1 + C.ab[2] * c.r2;
-            if (v > 0) D += real(2) * Phi - real(3) * c.p1 + c.p2;
-            const real y = X0 + (C.am[1] * R + C.am[2] * c.r1 + C.am[3] * c.r2);
-            A.Y[v][k] = v > 0 ? y - Phi : y;
+            D = fma(C.ab[2], c.r2, fma(C.ab[1], c.r1, mul_r(C.ab[0], R)));
+            real y = fma(C.am[3], c.r2, fma(C.am[2], c.r1, mul_r(C.am[1], R)));
+            if (v > 0) {
+                D = add_r(D, fma(real(2), Phi, fma(real(-3), c.p1, c.p2)));
+                y = sub_r(y, Phi);
+            } else {
+                y = add_r(X0, y);
+            }
+            A.Y[v][k] = y;
         }
         A.R0[v][k] = R;
         if (v > 0) A.F0[v][k] = Phi;
@@ -498,16 +508,14 @@ __device__ __forceinline__ real advance(const StencilArgs<real> &A, int v, real 
     }
     real D;
     if (kind == kEuler0) {
-        D = C.dt * R;
+        D = mul_r(C.dt, R);
         A.a[v][k] = Phi;
-    } else if (kind == kEuler1) {
-        D = C.dt * R + (Phi - c.a);
-        A.a[v][k] = C.ab[1] * R - real(3) * Phi;
     } else {
-        D = C.ab[0] * R + real(2) * Phi + (c.a + c.b);
-        A.a[v][k] = C.ab[1] * R - real(3) * Phi;
+        if (kind == kEuler1) D = add_r(mul_r(C.dt, R), sub_r(Phi, c.a));
+        else D = add_r(fma(real(2), Phi, mul_r(C.ab[0], R)), add_r(c.a, c.b));
+        A.a[v][k] = fma(real(-3), Phi, mul_r(C.ab[1], R));
     }
-    A.b[v][k] = C.ab[2] * R + Phi;
+    A.b[v][k] = fma(C.ab[2], R, Phi);
     return D;
 }
 
@@ -586,9 +594,10 @@ __device__ __forceinline__ void stage_tiles(const StageSpec<real> *sp, int tid)
 
 // Tile origin of a single-grid launch: the block index, which the compiler
 // re-reads where it needs it instead of keeping it in a register.
+template <int TY>
 struct GridOrigin {
     __device__ __forceinline__ int x0() const { return blockIdx.x * kTile; }
-    __device__ __forceinline__ int y0() const { return blockIdx.y * kTile; }
+    __device__ __forceinline__ int y0() const { return blockIdx.y * TY; }
 };
 
 // Tile origin of an ensemble launch: two ints in shared memory, loaded at
@@ -607,12 +616,12 @@ struct SharedOrigin {
 
 // Fluxes through faces f0 .. f1 - 1 of one row (kX: x-faces, r the row) or
 // one column (y-faces, r the column) of the staged tile.
-template <typename real, bool kX>
-__device__ __forceinline__ void sweep_faces(StencilSmem<real> &sm, const Coef<real> &C, int r, int f0, int f1)
+template <typename real, int TY, bool kX>
+__device__ __forceinline__ void sweep_faces(StencilSmem<real, TY> &sm, const Coef<real> &C, int r, int f0, int f1)
 {
     // strides along the sweep, and from a face's first corner to its second
     constexpr int sq = kX ? 1 : kStride, sc = kX ? 1 : kCornerStride, sc2 = kX ? kCornerStride : 1;
-    constexpr int sf = kX ? 1 : kTile, sv = kX ? kTile * (kTile + 1) : (kTile + 1) * kTile;
+    constexpr int sf = kX ? 1 : kTile, sv = kX ? TY * (kTile + 1) : (TY + 1) * kTile;
     const int o0 = (kX ? (r + kHalo) * kStride : r + kHalo) + f0 * sq;   // cell f0 - 2
     const real *pw = sm.w + o0, *pn = (kX ? sm.P : sm.Q) + o0, *pt = (kX ? sm.Q : sm.P) + o0;
     const real *cb = sm.Bc + (kX ? (r + 1) * kCornerStride : r + 1) + f0 * sc;   // face f0 - 1
@@ -647,11 +656,13 @@ __device__ __forceinline__ void sweep_faces(StencilSmem<real> &sm, const Coef<re
     }
 }
 
-// One 32 x 32 tile of one grid, at the origin O gives: the whole stencil stage.
-template <typename real, int kSpec, typename Origin>
+// One tile of one grid, 32 columns by TY rows at the origin O gives: the whole
+// stencil stage.
+template <typename real, int kSpec, int TY, typename Origin>
 __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const Origin &O, unsigned char *smem_raw)
 {
-    StencilSmem<real> &sm = *reinterpret_cast<StencilSmem<real> *>(smem_raw);
+    using S = StencilSmem<real, TY>;
+    S &sm = *reinterpret_cast<S *>(smem_raw);
     const Geo &G = A.geo;
     const int nx = G.nx, ny = G.ny;
     const int tid = threadIdx.x;
@@ -663,12 +674,12 @@ __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const O
     //         Corners: array index (corner + 1) in [0, nx + 2] x [0, ny + 2].
     {
         const StageSpec<real> spec[4] = {
-            {A.w_in, (size_t)G.px, O.x0() - kHalo, O.y0() - kHalo, kTileIn, kTileIn, nx, ny, sm.w, kStride, false},
-            {A.P_in, (size_t)G.px, O.x0() - kHalo, O.y0() - kHalo, kTileIn, kTileIn, nx, ny, sm.P, kStride, false},
-            {A.Qc_in, (size_t)G.py, O.y0() - kHalo, O.x0() - kHalo, kTileIn, kTileIn, ny, nx, sm.Q, kStride, true},
-            {A.Bc, (size_t)G.pc, O.x0(), O.y0(), kCorner, kCorner, nx + 3, ny + 3, sm.Bc, kCornerStride, false}};
-        // 36 x 18 pairs per state tile: at most 3 per thread
-        stage_tiles<real, 4, (kTileIn * (kTileIn / 2) + kStencilThreads - 1) / kStencilThreads>(spec, tid);
+            {A.w_in, (size_t)G.px, O.x0() - kHalo, O.y0() - kHalo, TY + 4, kTileIn, nx, ny, sm.w, kStride, false},
+            {A.P_in, (size_t)G.px, O.x0() - kHalo, O.y0() - kHalo, TY + 4, kTileIn, nx, ny, sm.P, kStride, false},
+            {A.Qc_in, (size_t)G.py, O.y0() - kHalo, O.x0() - kHalo, kTileIn, TY + 4, ny, nx, sm.Q, kStride, true},
+            {A.Bc, (size_t)G.pc, O.x0(), O.y0(), TY + 3, kCorner, nx + 3, ny + 3, sm.Bc, kCornerStride, false}};
+        // at 32 rows, 36 x 18 pairs per state tile: at most 3 per thread
+        stage_tiles<real, 4, ((TY + 4) * (kTileIn / 2) + kStencilThreads - 1) / kStencilThreads>(spec, tid);
     }
     if (tid < kTile) sm.colbits[tid] = 0u;
     __syncthreads();
@@ -683,10 +694,10 @@ __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const O
     // ---- 2. ghost layers (Sec. 2.4): x-sides over interior rows, then
     //         y-sides over every column, so corners come by composition.
     const bool westT = O.x0() == 0, eastT = O.x0() + kTile + kHalo > nx;
-    const bool southT = O.y0() == 0, northT = O.y0() + kTile + kHalo > ny;
+    const bool southT = O.y0() == 0, northT = O.y0() + TY + kHalo > ny;
     if (westT || eastT) {
-        for (int k = tid; k < 4 * (kTileIn - 2); k += kStencilThreads) {
-            int ty = 1 + k % (kTileIn - 2), which = k / (kTileIn - 2);   // ty in [1, 35)
+        for (int k = tid; k < 4 * (TY + 2); k += kStencilThreads) {
+            int ty = 1 + k % (TY + 2), which = k / (TY + 2);
             int gy = O.y0() - kHalo + ty;
             if (gy < 0 || gy >= ny) continue;
             int side = which < 2 ? 0 : 1, kk = which & 1;
@@ -718,7 +729,7 @@ __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const O
             if ((side == 2 && !southT) || (side == 3 && !northT)) continue;
             int gy = side == 2 ? -1 - kk : ny + kk;
             int ty = gy - O.y0() + kHalo;
-            if (ty < 0 || ty >= kTileIn) continue;
+            if (ty < 0 || ty >= TY + 4) continue;
             int sy = side == 2 ? kk : ny - 1 - kk;
             int sty = sy - O.y0() + kHalo;
             int gi = ty * kStride + tx, si = sty * kStride + tx;
@@ -735,23 +746,35 @@ __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const O
         }
     }
     // ---- 3. still-water depth d (Sec. 2.1) on the tile + 1 ring
-    for (int k = tid; k < kDcell * kDcell; k += kStencilThreads) {
+    for (int k = tid; k < kDcell * (TY + 2); k += kStencilThreads) {
         int cy = k / kDcell, cx = k % kDcell;
         sm.d[cy * kDStride + cx] = cell_d(cx, cy);
     }
     __syncthreads();
 
     // ---- 4. fluxes through every face of the tile, each computed once.
-    //         Warps 0-3 sweep x-faces, warps 4-7 y-faces; a lane owns one
-    //         row (x) or column (y) and 8 consecutive faces of it (the last
-    //         warp of each half also face 32), so every cell is reconstructed
-    //         once per direction: the right cell of a face is the left cell
-    //         of the next.
-    {
+    //         At 32 rows warps 0-3 sweep x-faces, warps 4-7 y-faces; a lane
+    //         owns one row (x) or column (y) and 8 consecutive faces of it
+    //         (the last warp of each half also face 32), so every cell is
+    //         reconstructed once per direction: the right cell of a face is
+    //         the left cell of the next.  At fewer rows a thread takes one
+    //         face at a time.
+    if constexpr (TY == kTile) {
         const int lane = tid & 31, wq = (tid >> 5) & 3;
         const int f0 = wq * 8, f1 = wq == 3 ? kTile + 1 : f0 + 8;
-        if (tid < 4 * 32) sweep_faces<real, true>(sm, C, lane, f0, f1);
-        else sweep_faces<real, false>(sm, C, lane, f0, f1);
+        if (tid < 4 * 32) sweep_faces<real, TY, true>(sm, C, lane, f0, f1);
+        else sweep_faces<real, TY, false>(sm, C, lane, f0, f1);
+    } else {
+        constexpr int nxf = TY * (kTile + 1), nx32 = (nxf + 31) / 32 * 32, nyf = (TY + 1) * kTile;
+        for (int k = tid; k < nx32 + nyf; k += kStencilThreads) {
+            if (k < nxf) {
+                const int r = k / (kTile + 1), f = k - r * (kTile + 1);
+                sweep_faces<real, TY, true>(sm, C, r, f, f + 1);
+            } else if (k >= nx32) {
+                const int f = (k - nx32) / kTile, c = (k - nx32) % kTile;
+                sweep_faces<real, TY, false>(sm, C, c, f, f + 1);
+            }
+        }
     }
     __syncthreads();
 
@@ -763,11 +786,10 @@ __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const O
     // the sponge (Eq. 30) on the last stage, where the tile reaches into one
     const bool sponge_tile = A.final_stage &&
                              (O.x0() < C.spw[0] || O.x0() + kTile > nx - C.spw[1] || O.y0() < C.spw[2] ||
-                              O.y0() + kTile > ny - C.spw[3]);
-    constexpr int kRows = kTile / (kStencilThreads / 32);   // rows per thread
+                              O.y0() + TY > ny - C.spw[3]);
 #pragma unroll 1
-    for (int rr = 0; rr < kRows; rr++) {
-        const int cx = lane, cy = (tid >> 5) + rr * (kStencilThreads / 32);
+    for (int cy = tid >> 5; cy < TY; cy += kStencilThreads / 32) {
+        const int cx = lane;
         const int i = O.x0() + cx, j = O.y0() + cy;
         const bool valid = i < nx && j < ny;
         const int o = (cy + kHalo) * kStride + cx + kHalo;
@@ -785,60 +807,65 @@ __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const O
         real c00 = cb[0], c10 = cb[1], c01 = cb[kCornerStride], c11 = cb[kCornerStride + 1];
         const real Bb = cell_bbar(c00, c10, c01, c11);
         real w0 = sm.w[o], P0 = sm.P[o], Q0 = sm.Q[o];
-        const real hb = w0 - Bb;
-        const real E = (sm.Fx[0][cy][cx] - sm.Fx[0][cy][cx + 1]) * rdx + (sm.Fy[0][cy][cx] - sm.Fy[0][cy + 1][cx]) * rdy;
-        real F = (sm.Fx[1][cy][cx] - sm.Fx[1][cy][cx + 1]) * rdx + (sm.Fy[1][cy][cx] - sm.Fy[1][cy + 1][cx]) * rdy;
-        real Gq = (sm.Fx[2][cy][cx] - sm.Fx[2][cy][cx + 1]) * rdx + (sm.Fy[2][cy][cx] - sm.Fy[2][cy + 1][cx]) * rdy;
+        const real hb = sub_r(w0, Bb);
+        auto div = [&](int v) {
+            return fma(sub_r(sm.Fx[v][cy][cx], sm.Fx[v][cy][cx + 1]), rdx,
+                       mul_r(sub_r(sm.Fy[v][cy][cx], sm.Fy[v][cy + 1][cx]), rdy));
+        };
+        const real E = div(0);
         // bed slope: the face beds' difference is half that of the corner sums
-        F -= hb * C.hgx * ((c10 + c11) - (c00 + c01));
-        Gq -= hb * C.hgy * ((c01 + c11) - (c00 + c10));
+        const real sx = sub_r(add_r(c10, c11), add_r(c00, c01)), sy = sub_r(add_r(c01, c11), add_r(c00, c10));
+        real F = fma(mul_r(hb, -C.hgx), sx, div(1));
+        real Gq = fma(mul_r(hb, -C.hgy), sy, div(2));
         if (friction != kFricNone) {   // Eq. 31-32 with the Eq. 14 device
-            const real fm = friction_depth(friction, C.fric, hb, eps, C.hwet) * sqrt_r(P0 * P0 + Q0 * Q0);
-            F -= fm * P0;
-            Gq -= fm * Q0;
+            const real fm = mul_r(friction_depth(friction, C.fric, hb, eps, C.hwet),
+                                  sqrt_r(fma(P0, P0, mul_r(Q0, Q0))));
+            F = fma(-fm, P0, F);
+            Gq = fma(-fm, Q0, Gq);
         }
         real Fs = real(0), Gs = real(0);
         const int od = (cy + 1) * kDStride + cx + 1;
         const real dd = sm.d[od];
         if (bsnq) {
-            const real dDx = sm.d[od + 1] - sm.d[od - 1], dDy = sm.d[od + kDStride] - sm.d[od - kDStride];
-            const real d2 = dd * dd;
+            const real dDx = sub_r(sm.d[od + 1], sm.d[od - 1]), dDy = sub_r(sm.d[od + kDStride], sm.d[od - kDStride]);
+            const real d2 = mul_r(dd, dd);
             const real *W = sm.w + o;
             const int S1 = kStride, S2 = 2 * kStride;
-            // eta = w - w_s enters only through differences, where w_s cancels
-            const real e00 = w0;
+            // undivided differences; eta = w - w_s enters only through them, where w_s cancels
+            const real two = real(2);
             const real eE = W[1], eW = W[-1], eN = W[S1], eS = W[-S1];
             const real eNE = W[S1 + 1], eNW = W[S1 - 1], eSE = W[-S1 + 1], eSW = W[-S1 - 1];
-            const real pN = eNE - eNW, pS = eSE - eSW;             // x-differences of the rows above and below
-            const real gx = eE - eW, gy = eN - eS;
-            const real exy = (pN - pS) * C.rdxdy4;
-            const real exx = (eE - real(2) * e00 + eW) * C.rdx2;
-            const real eyy = (eN - real(2) * e00 + eS) * C.rdy2;
-            const real exxx = (W[2] - W[-2]) - real(2) * gx;
-            const real eyyy = (W[S2] - W[-S2]) - real(2) * gy;
-            const real exyy = (pN + pS) - real(2) * gx;
-            const real exxy = ((eNE - eSE) + (eNW - eSW)) - real(2) * gy;
-            const real ddx = dDx * C.hrdx, ddy = dDy * C.hrdy;
-            const real K2 = C.Bdg * d2;
-            F += K2 * (dd * (exxx * C.rdx3h + exyy * C.rdxdy2h) + ddx * (real(2) * exx + eyy) + ddy * exy);
-            Gq += K2 * (dd * (eyyy * C.rdy3h + exxy * C.rdx2dyh) + ddy * (real(2) * eyy + exx) + ddx * exy);
+            const real pN = sub_r(eNE, eNW), pS = sub_r(eSE, eSW);   // of the rows above and below
+            const real gx = sub_r(eE, eW), gy = sub_r(eN, eS);
+            const real exy = mul_r(real(0.25), sub_r(pN, pS));
+            const real exx = add_r(fma(-two, w0, eE), eW), eyy = add_r(fma(-two, w0, eN), eS);
+            const real exxx = fma(-two, gx, sub_r(W[2], W[-2])), eyyy = fma(-two, gy, sub_r(W[S2], W[-S2]));
+            const real exyy = fma(-two, gx, add_r(pN, pS));
+            const real exxy = fma(-two, gy, add_r(sub_r(eNE, eSE), sub_r(eNW, eSW)));
+            // K d^2 / (2 dx) [A (d exxx + 2 d_x exx) + B (d exyy + d_x eyy + d_y exy / 4)], A = 1/dx^2, B = 1/dy^2
+            const real x1 = fma(add_r(dDx, dDx), exx, mul_r(dd, exxx));
+            const real x2 = fma(dDy, exy, fma(dDx, eyy, mul_r(dd, exyy)));
+            const real y1 = fma(add_r(dDy, dDy), eyy, mul_r(dd, eyyy));
+            const real y2 = fma(dDx, exy, fma(dDy, exx, mul_r(dd, exxy)));
+            F = fma(mul_r(d2, C.Kx), fma(C.rdy2, x2, mul_r(C.rdx2, x1)), F);
+            Gq = fma(mul_r(d2, C.Ky), fma(C.rdx2, y2, mul_r(C.rdy2, y1)), Gq);
             const real *Pt = sm.P + o, *Qt = sm.Q + o;
-            const real m1 = dd * dDx * C.c6, m2 = dd * dDy * C.c6, m3 = C.B3xy * d2;
-            Fs = m1 * (Qt[S1] - Qt[-S1]) + m2 * (Qt[1] - Qt[-1]) +
-                 m3 * ((Qt[S1 + 1] - Qt[-S1 + 1]) - (Qt[S1 - 1] - Qt[-S1 - 1]));
-            Gs = m2 * (Pt[1] - Pt[-1]) + m1 * (Pt[S1] - Pt[-S1]) +
-                 m3 * ((Pt[S1 + 1] - Pt[-S1 + 1]) - (Pt[S1 - 1] - Pt[-S1 - 1]));
+            const real dc = mul_r(dd, C.c6), m1 = mul_r(dc, dDx), m2 = mul_r(dc, dDy), m3 = mul_r(C.B3xy, d2);
+            Fs = fma(m3, sub_r(sub_r(Qt[S1 + 1], Qt[-S1 + 1]), sub_r(Qt[S1 - 1], Qt[-S1 - 1])),
+                     fma(m2, sub_r(Qt[1], Qt[-1]), mul_r(m1, sub_r(Qt[S1], Qt[-S1]))));
+            Gs = fma(m3, sub_r(sub_r(Pt[S1 + 1], Pt[-S1 + 1]), sub_r(Pt[S1 - 1], Pt[-S1 - 1])),
+                     fma(m1, sub_r(Pt[S1], Pt[-S1]), mul_r(m2, sub_r(Pt[1], Pt[-1]))));
         }
         real w1 = w0, dU = real(0), dV = real(0);
         if (valid) {
             real dw = advance<real, kSpec>(A, 0, w0, E, real(0), kr, cw);
-            w1 = stage_kind<kSpec>(A) == kAM4 ? dw : w0 + dw;   // the AM4 base of w holds w^n
+            w1 = stage_kind<kSpec>(A) == kAM4 ? dw : add_r(w0, dw);   // the AM4 base of w holds w^n
             dU = advance<real, kSpec>(A, 1, real(0), F, Fs, kr, cu);
             dV = advance<real, kSpec>(A, 2, real(0), Gq, Gs, kr, cv);
             if (w1 < Bb) w1 = Bb;   // Reading A-D1
             if (sponge_tile) {
                 real gam = sponge_gamma<real>(C, G, i, j);
-                if (gam < real(1) && dd > real(0)) w1 = ws + gam * (w1 - ws);
+                if (gam < real(1) && dd > real(0)) w1 = fma(gam, sub_r(w1, ws), ws);
             }
             A.w_out[kr] = w1;
             A.U_out[kr] = dU;
@@ -850,20 +877,30 @@ __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const O
         sm.Vout[cy][cx] = dV;
     }
     __syncthreads();
-    for (int k = tid; k < kTile * kTile; k += kStencilThreads) {
-        int c = k / kTile, r = k % kTile;
+    for (int k = tid; k < kTile * TY; k += kStencilThreads) {
+        int c = k / TY, r = k % TY;
         int i = O.x0() + c, j = O.y0() + r;
         if (i < nx && j < ny) A.Vc_out[(size_t)i * G.py + j] = sm.Vout[r][c];
     }
-    if (tid < kTile && O.x0() + tid < nx) A.mask_c[(size_t)(O.x0() + tid) * G.nwy + (O.y0() >> 5)] = sm.colbits[tid];
+    if (tid < kTile && O.x0() + tid < nx) {
+        uint32_t *word = A.mask_c + (size_t)(O.x0() + tid) * G.nwy + (O.y0() >> 5);
+        if constexpr (TY == 32) {
+            *word = sm.colbits[tid];
+        } else {   // the tile's own bits of a word it shares
+            const int sh = O.y0() & 31;
+            const uint32_t own = ((1u << TY) - 1u) << sh, bits = sm.colbits[tid] << sh;
+            if (bits != own) atomicAnd(word, ~own | bits);
+            if (bits) atomicOr(word, bits);
+        }
+    }
 }
 
-template <int kSpec>
+template <int kSpec, int TY>
 __global__ void __launch_bounds__(kStencilThreads, 2) k_stencil(const __grid_constant__ StencilArgs<double> A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     dependent_launch_wait_then_release();
-    stencil_tile<double, kSpec>(A, GridOrigin(), smem_raw);
+    stencil_tile<double, kSpec, TY>(A, GridOrigin<TY>(), smem_raw);
 }
 
 // FP32 (celeris_stencil_f32.cuh): 64 columns and 4 kR rows per block.
@@ -915,7 +952,7 @@ __global__ void __launch_bounds__(kStencilThreads, 2)
     }
     load_args(A, args + d.x);
     __syncthreads();
-    stencil_tile<double, kSpec>(A, SharedOrigin{origin}, smem_raw);
+    stencil_tile<double, kSpec, kTile>(A, SharedOrigin{origin}, smem_raw);
 }
 
 template <int kSpec>
@@ -1825,7 +1862,7 @@ __device__ __noinline__ void persist_tile(const StencilArgs<double> &__restrict_
                                           unsigned char *smem_raw)
 {
     __builtin_assume(__isShared(&A));
-    stencil_tile<double, kSpec>(A, SharedOrigin{origin}, smem_raw);
+    stencil_tile<double, kSpec, kTile>(A, SharedOrigin{origin}, smem_raw);
 }
 
 // FP32: each half of the block takes a tile of its own (kPThreads threads).
@@ -1861,7 +1898,7 @@ __device__ __forceinline__ void persist_flag(unsigned *bar, unsigned code, unsig
 template <typename real>
 __host__ __device__ constexpr size_t persist_smem()
 {
-    return sizeof(real) == 4 ? (kStencilThreads / kPThreads) * sizeof(PairSmem<kPairRows>) : sizeof(StencilSmem<double>);
+    return sizeof(real) == 4 ? (kStencilThreads / kPThreads) * sizeof(PairSmem<kPairRows>) : sizeof(StencilSmem<double, kTile>);
 }
 
 template <typename real>
@@ -2151,22 +2188,39 @@ cudaError_t launch_ghost_table(const Geo &g, const Phys &p, const Bnd &b, const 
     return cudaGetLastError();
 }
 
-template <>
-cudaError_t launch_stencil<double>(const StencilArgs<double> &a, cudaStream_t st)
+namespace {
+
+template <int TY>
+cudaError_t launch_stencil_rows(const StencilArgs<double> &a, cudaStream_t st)
 {
     static bool configured[3] = {false, false, false};
-    const size_t smem = sizeof(StencilSmem<double>);
+    constexpr size_t smem = sizeof(StencilSmem<double, TY>);
     const int spec = stencil_spec(a);
-    auto *kern = spec == 1 ? k_stencil<1> : spec == 2 ? k_stencil<2> : k_stencil<0>;
+    auto *kern = spec == 1 ? k_stencil<1, TY> : spec == 2 ? k_stencil<2, TY> : k_stencil<0, TY>;
     if (!configured[spec]) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         configured[spec] = true;
     }
-    dim3 grid((a.geo.nx + kTile - 1) / kTile, (a.geo.ny + kTile - 1) / kTile);
+    dim3 grid((a.geo.nx + kTile - 1) / kTile, (a.geo.ny + TY - 1) / TY);
     cudaError_t e = launch_step_kernel(kern, grid, dim3(kStencilThreads), smem, st, a);
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+}  // namespace
+
+template <>
+cudaError_t launch_stencil<double>(const StencilArgs<double> &a, cudaStream_t st)
+{
+    const long tiles = (long)((a.geo.nx + kTile - 1) / kTile) * ((a.geo.ny + kTile - 1) / kTile);
+    // Rows per tile: the FP64 pipes are the bound, so what counts on a small
+    // grid is that every SM has work.  Step in us with 32 / 4 / 2 rows:
+    // 1024 x 1024 (1024 tiles of 32 x 32) 1762 / 1928 / 2135; 512 x 512 (256)
+    // 586 / 537 / 577; 200 x 150 (35) 311 / 123 / 133; 128 x 128 (16) 297 / 83
+    // / 87; 256 x 32 (8) 305 / 83 / 70.
+    if (tiles >= 512) return launch_stencil_rows<kTile>(a, st);
+    if (tiles >= 16) return launch_stencil_rows<4>(a, st);
+    return launch_stencil_rows<2>(a, st);
 }
 
 namespace {
@@ -2240,7 +2294,7 @@ cudaError_t launch_stencil_batch(const StencilArgs<real> *args, const int2 *desc
         threads = kPThreads;
     } else {
         kern = spec == 1 ? k_stencil_batch<1> : spec == 2 ? k_stencil_batch<2> : k_stencil_batch<0>;
-        smem = sizeof(StencilSmem<double>);
+        smem = sizeof(StencilSmem<double, kTile>);
         threads = kStencilThreads;
     }
     if (!configured[spec]) {

@@ -233,12 +233,12 @@ __device__ __forceinline__ void fix_pair(pk w, pk Blo, pk Bhi, pk &lo, pk &hi, p
     auto fix = [](float w, float bl, float bh, float &wl, float &wh, float &l, float &h) {
         if (h < 0.f) {
             wh = bh;
-            wl = 2.f * w - bh;
+            wl = fma(2.f, w, -bh);
             h = 0.f;
             l = fmaxf(wl - bl, 0.f);
         } else if (l < 0.f) {
             wl = bl;
-            wh = 2.f * w - bl;
+            wh = fma(2.f, w, -bl);
             l = 0.f;
             h = fmaxf(wh - bh, 0.f);
         }
@@ -862,11 +862,11 @@ __device__ __forceinline__ void stencil_tile_pair(const StencilArgs<float> &A, c
             un(dd, d0, d1);
             if (ok0) {
                 const float gam = sponge_gamma<float>(C, G, i, j);
-                if (gam < 1.f && d0 > 0.f) a = ws + gam * (a - ws);
+                if (gam < 1.f && d0 > 0.f) a = fma(gam, sub_r(a, ws), ws);
             }
             if (ok1) {
                 const float gam = sponge_gamma<float>(C, G, i + 1, j);
-                if (gam < 1.f && d1 > 0.f) b = ws + gam * (b - ws);
+                if (gam < 1.f && d1 > 0.f) b = fma(gam, sub_r(b, ws), ws);
             }
         }
         if (ok0) {
