@@ -221,30 +221,15 @@ __device__ __forceinline__ void face_flux(const Dual<T> w[4], const Dual<T> P[4]
 // argument when equal, fmin too, sqrt has derivative 0 at 0), then the
 // adjoints back through every operation.  Outputs: the adjoints of the 4
 // cells' (w, P, Q) and of the three face beds (Bm, Bf, Bp), added to.
+// adjoint ls of four times the half slope (minmod_choice's value) into its
+// three cells: the candidates are 2 theta (q0 - qm), qp - qm, 2 theta (qp - q0)
 template <typename T>
-__device__ __forceinline__ int minmod3_sel(T th, T qm, T q0, T qp)
+__device__ __forceinline__ void slope_vjp(int sel, T th2, T ls, T &lqm, T &lq0, T &lqp)
 {
-    const T a = th * (q0 - qm), b = T(0.5) * (qp - qm), c = th * (qp - q0);
-    const int ilo_bc = b <= c ? 2 : 3, ihi_bc = b >= c ? 2 : 3;
-    const T lo_bc = b <= c ? b : c, hi_bc = b >= c ? b : c;
-    const int ilo = a <= lo_bc ? 1 : ilo_bc, ihi = a >= hi_bc ? 1 : ihi_bc;
-    const T lo = a <= lo_bc ? a : lo_bc, hi = a >= hi_bc ? a : hi_bc;
-    return lo > T(0) ? ilo : (hi < T(0) ? ihi : 0);
-}
-
-template <typename T>
-__device__ __forceinline__ T slope_of(int sel, T th, T qm, T q0, T qp)
-{
-    return sel == 1 ? th * (q0 - qm) : sel == 2 ? T(0.5) * (qp - qm) : sel == 3 ? th * (qp - q0) : T(0);
-}
-
-// adjoint ls of the selected slope into its three cells
-template <typename T>
-__device__ __forceinline__ void slope_vjp(int sel, T th, T ls, T &lqm, T &lq0, T &lqp)
-{
-    if (sel == 1) { lqm -= th * ls; lq0 += th * ls; }
-    else if (sel == 2) { lqm -= T(0.5) * ls; lqp += T(0.5) * ls; }
-    else if (sel == 3) { lq0 -= th * ls; lqp += th * ls; }
+    const T v = sel == 2 ? ls : th2 * ls;
+    if (sel == 1) { lqm -= v; lq0 += v; }
+    else if (sel == 2) { lqm -= v; lqp += v; }
+    else if (sel == 3) { lq0 -= v; lqp += v; }
 }
 
 // dk/dh of desing (Eq. 14) with its branch of max(h^4, eps)
@@ -258,65 +243,91 @@ __device__ __forceinline__ T desing_dh(T h, T eps)
 }
 
 template <typename T>
-__device__ __forceinline__ void face_flux_vjp(const T w[4], const T P[4], const T Q[4], T Bm, T Bf, T Bp, T th, T g,
-                                              T eps, int dir, const T lH[3], T lw[4], T lP[4], T lQ[4], T lB[3])
+__device__ __forceinline__ void face_flux_vjp(const T w[4], const T P[4], const T Q[4], T Bm, T Bf, T Bp, T th2, T g,
+                                              T eps, T hwet, int dir, const T lH[3], T lw[4], T lP[4], T lQ[4], T lB[3])
 {
-    // reconstruction: left cell 1 (its high face), right cell 2 (its low face)
+    // reconstruction: left cell 1 (its high face), right cell 2 (its low
+    // face), in the stencil's form (FaceSweep)
     int sw[2], sP[2], sQ[2], fix[2];   // fix: 0 none, 1 high face clamped, 2 low face clamped
     T f[2][3];                          // hiL and loR in (w, P, Q)
+    T dep[2];                           // w less the face bed, before it is held at 0
 #pragma unroll
     for (int c = 0; c < 2; c++) {
-        const T Blo = c == 0 ? Bm : Bf, Bhi = c == 0 ? Bf : Bp;
-        sw[c] = minmod3_sel(th, w[c], w[c + 1], w[c + 2]);
-        sP[c] = minmod3_sel(th, P[c], P[c + 1], P[c + 2]);
-        sQ[c] = minmod3_sel(th, Q[c], Q[c + 1], Q[c + 2]);
-        const T s0 = slope_of(sw[c], th, w[c], w[c + 1], w[c + 2]);
-        const T lo0 = w[c + 1] - T(0.5) * s0, hi0 = w[c + 1] + T(0.5) * s0;
-        fix[c] = hi0 < Bhi ? 1 : (lo0 < Blo ? 2 : 0);
-        const T v0 = c == 0 ? (fix[c] == 1 ? Bhi : fix[c] == 2 ? T(2) * w[1] - Blo : hi0)
-                            : (fix[c] == 1 ? T(2) * w[2] - Bhi : fix[c] == 2 ? Blo : lo0);
-        const T sgn = c == 0 ? T(0.5) : T(-0.5);
-        f[c][0] = v0;
-        f[c][1] = P[c + 1] + sgn * slope_of(sP[c], th, P[c], P[c + 1], P[c + 2]);
-        f[c][2] = Q[c + 1] + sgn * slope_of(sQ[c], th, Q[c], Q[c + 1], Q[c + 2]);
+        const T Blo = c == 0 ? Bm : Bf, Bhi = c == 0 ? Bf : Bp, q4 = c == 0 ? T(0.25) : T(-0.25);
+        T m;
+        sP[c] = minmod_choice(th2 * (P[c + 1] - P[c]), P[c + 2] - P[c], th2 * (P[c + 2] - P[c + 1]), m);
+        f[c][1] = P[c + 1] + q4 * m;
+        sQ[c] = minmod_choice(th2 * (Q[c + 1] - Q[c]), Q[c + 2] - Q[c], th2 * (Q[c + 2] - Q[c + 1]), m);
+        f[c][2] = Q[c + 1] + q4 * m;
+        sw[c] = minmod_choice(th2 * (w[c + 1] - w[c]), w[c + 2] - w[c], th2 * (w[c + 2] - w[c + 1]), m);
+        const T lo0 = w[c + 1] - T(0.25) * m, hi0 = w[c + 1] + T(0.25) * m;
+        const T dlo = lo0 - Blo, dhi = hi0 - Bhi;
+        fix[c] = below_zero(dhi) ? 1 : (below_zero(dlo) ? 2 : 0);
+        f[c][0] = c == 0 ? hi0 : lo0;
+        dep[c] = c == 0 ? dhi : dlo;
+        if (fix[c]) {
+            f[c][0] = c == 0 ? (fix[c] == 1 ? Bhi : T(2) * w[1] - Blo) : (fix[c] == 1 ? T(2) * w[2] - Bhi : Blo);
+            dep[c] = f[c][0] - Bf;
+        }
     }
     // central-upwind flux on (w, normal, tangential)
     const int nv = dir == 0 ? 1 : 2, tv = dir == 0 ? 2 : 1;
     const T wL = f[0][0], nL = f[0][nv], tL = f[0][tv], wR = f[1][0], nR = f[1][nv], tR = f[1][tv];
-    const T aL = wL - Bf, aR = wR - Bf;
-    const bool pL = aL >= T(0), pR = aR >= T(0);
-    const T hL = pL ? aL : T(0), hR = pR ? aR : T(0);
-    const T kL = desing(hL, eps), kR = desing(hR, eps);
+    const bool pL = not_below(dep[0]), pR = not_below(dep[1]);
+    const T hL = pL ? dep[0] : T(0), hR = pR ? dep[1] : T(0);
+    // where both depths reach eps^(1/4), u = n / h and h u = n (Eq. 14's
+    // factor is 1/h there); cL, cR: d(celerity)/dh
+    const bool wet = at_least(hL, hwet) && at_least(hR, hwet);
+    const T ghL = g * hL, ghR = g * hR;
+    T kL, kR, sL, sR, cL, cR, qnL = nL, qtL = tL, qnR = nR, qtR = tR;
+    if (wet) {
+        const T rL = rsqrt_r(ghL), rR = rsqrt_r(ghR);
+        sL = ghL * rL;
+        sR = ghR * rR;
+        kL = g * rL * rL;
+        kR = g * rR * rR;
+        cL = T(0.5) * g * rL;
+        cR = T(0.5) * g * rR;
+    } else {
+        kL = desing(hL, eps);
+        kR = desing(hR, eps);
+        sL = sqrt(ghL);
+        sR = sqrt(ghR);
+        cL = sL > T(0) ? g / (T(2) * sL) : T(0);
+        cR = sR > T(0) ? g / (T(2) * sR) : T(0);
+    }
     const T uL = kL * nL, vL = kL * tL, uR = kR * nR, vR = kR * tR;
-    const T qnL = hL * uL, qtL = hL * vL, qnR = hR * uR, qtR = hR * vR;
-    const T sL = sqrt(g * hL), sR = sqrt(g * hR);
+    if (!wet) {
+        qnL = hL * uL;
+        qtL = hL * vL;
+        qnR = hR * uR;
+        qtR = hR * vR;
+    }
     const T ap1c = uL + sL, ap2c = uR + sR, am1c = uL - sL, am2c = uR - sR;
-    const bool apL = ap1c >= ap2c, amL = am1c <= am2c;
+    const bool apL = ge_r(ap1c, ap2c), amL = ge_r(am2c, am1c);
     const T ap1 = apL ? ap1c : ap2c, am1 = amL ? am1c : am2c;
-    const bool apK = ap1 >= T(0), amK = am1 <= T(0);
+    const bool apK = not_below(ap1), amK = !above_zero(am1);
     const T ap = apK ? ap1 : T(0), am = amK ? am1 : T(0);
     const T den = ap - am;
-    if (!(den > T(0))) return;
-    const T inv = T(1) / den, apam = ap * am;
-    const T FL1 = qnL * uL + T(0.5) * g * hL * hL, FR1 = qnR * uR + T(0.5) * g * hR * hR;
-    const T N0 = ap * qnL - am * qnR + apam * (wR - wL);
-    const T N1 = ap * FL1 - am * FR1 + apam * (qnR - qnL);
-    const T N2 = ap * (qnL * vL) - am * (qnR * vR) + apam * (qtR - qtL);
+    if (!above_zero(den)) return;
+    const T inv = rcp_r(den), apam = ap * am;
+    const T FL1 = qnL * uL + T(0.5) * (ghL * hL), FR1 = qnR * uR + T(0.5) * (ghR * hR);
+    const T FL2 = qnL * vL, FR2 = qnR * vR;
+    const T dw = wR - wL, dn = qnR - qnL, dt = qtR - qtL;
+    const T N0 = ap * qnL - am * qnR + apam * dw;
+    const T N1 = ap * FL1 - am * FR1 + apam * dn;
+    const T N2 = ap * FL2 - am * FR2 + apam * dt;
     // reverse
     const T lN0 = lH[0] * inv, lN1 = lH[1] * inv, lN2 = lH[2] * inv;
-    const T lden = -(lH[0] * N0 + lH[1] * N1 + lH[2] * N2) * inv * inv;
-    const T lapam = lN0 * (wR - wL) + lN1 * (qnR - qnL) + lN2 * (qtR - qtL);
-    const T lap = lN0 * qnL + lN1 * FL1 + lN2 * (qnL * vL) + lapam * am + lden;
-    const T lam = -(lN0 * qnR) - lN1 * FR1 - lN2 * (qnR * vR) + lapam * ap - lden;
-    const T lFL1 = lN1 * ap, lFR1 = -(lN1 * am);
-    T lqnL = lN0 * ap - lN1 * apam + lN2 * ap * vL + lFL1 * uL;
-    T lqnR = -(lN0 * am) + lN1 * apam - lN2 * am * vR + lFR1 * uR;
+    const T lden = -(lN0 * N0 + lN1 * N1 + lN2 * N2) * inv;
+    const T lapam = lN0 * dw + lN1 * dn + lN2 * dt;
+    const T lap = lN0 * qnL + lN1 * FL1 + lN2 * FL2 + lapam * am + lden;
+    const T lam = lapam * ap - (lN0 * qnR + lN1 * FR1 + lN2 * FR2) - lden;
+    const T lFL1 = lN1 * ap, lFR1 = -(lN1 * am), x0 = lN0 * apam, x1 = lN1 * apam, x2 = lN2 * apam;
+    const T lqnL = ap * (lN0 + lN1 * uL + lN2 * vL) - x1, lqnR = x1 - am * (lN0 + lN1 * uR + lN2 * vR);
     T lvL = lN2 * ap * qnL, lvR = -(lN2 * am * qnR);
-    const T lqtL = -(lN2 * apam), lqtR = lN2 * apam;
-    T lwL = -(lN0 * apam), lwR = lN0 * apam;
     T luL = lFL1 * qnL, luR = lFR1 * qnR;
-    T lhL = lFL1 * g * hL, lhR = lFR1 * g * hR;
-    T lsL = T(0), lsR = T(0);
+    T lhL = lFL1 * ghL, lhR = lFR1 * ghR, lsL = T(0), lsR = T(0);
     if (apK) {
         if (apL) { luL += lap; lsL += lap; }
         else { luR += lap; lsR += lap; }
@@ -325,45 +336,55 @@ __device__ __forceinline__ void face_flux_vjp(const T w[4], const T P[4], const 
         if (amL) { luL += lam; lsL -= lam; }
         else { luR += lam; lsR -= lam; }
     }
-    if (sL > T(0)) lhL += lsL * g / (T(2) * sL);
-    if (sR > T(0)) lhR += lsR * g / (T(2) * sR);
-    lhL += lqnL * uL + lqtL * vL;
-    luL += lqnL * hL;
-    lvL += lqtL * hL;
-    lhR += lqnR * uR + lqtR * vR;
-    luR += lqnR * hR;
-    lvR += lqtR * hR;
-    const T lkL = luL * nL + lvL * tL, lkR = luR * nR + lvR * tR;
+    lhL += lsL * cL;
+    lhR += lsR * cR;
     T lf[2][3];
-    lf[0][nv] = luL * kL;
-    lf[0][tv] = lvL * kL;
-    lf[1][nv] = luR * kR;
-    lf[1][tv] = lvR * kR;
-    lhL += lkL * desing_dh(hL, eps);
-    lhR += lkR * desing_dh(hR, eps);
+    if (wet) {
+        const T gL = luL * nL + lvL * tL, gR = luR * nR + lvR * tR;
+        lhL -= gL * kL * kL;
+        lhR -= gR * kR * kR;
+        lf[0][nv] = luL * kL + lqnL;
+        lf[0][tv] = lvL * kL - x2;
+        lf[1][nv] = luR * kR + lqnR;
+        lf[1][tv] = lvR * kR + x2;
+    } else {
+        lhL += lqnL * uL - x2 * vL;
+        luL += lqnL * hL;
+        lvL -= x2 * hL;
+        lhR += lqnR * uR + x2 * vR;
+        luR += lqnR * hR;
+        lvR += x2 * hR;
+        lhL += (luL * nL + lvL * tL) * desing_dh(hL, eps);
+        lhR += (luR * nR + lvR * tR) * desing_dh(hR, eps);
+        lf[0][nv] = luL * kL;
+        lf[0][tv] = lvL * kL;
+        lf[1][nv] = luR * kR;
+        lf[1][tv] = lvR * kR;
+    }
     const T laL = pL ? lhL : T(0), laR = pR ? lhR : T(0);
-    lf[0][0] = lwL + laL;
-    lf[1][0] = lwR + laR;
+    lf[0][0] = laL - x0;
+    lf[1][0] = laR + x0;
     lB[1] -= laL + laR;
     // reconstruction reversed
 #pragma unroll
     for (int c = 0; c < 2; c++) {
-        const T sgn = c == 0 ? T(0.5) : T(-0.5);
+        const T q4 = c == 0 ? T(0.25) : T(-0.25);
         const T lv = lf[c][0];
         const int bl = c == 0 ? 0 : 1, bh = c == 0 ? 1 : 2;   // indices of Blo, Bhi in lB
-        if (c == 0) {
+        if (fix[c] == 0) {
+            lw[c + 1] += lv;
+            slope_vjp(sw[c], th2, q4 * lv, lw[c], lw[c + 1], lw[c + 2]);
+        } else if (c == 0) {
             if (fix[c] == 1) lB[bh] += lv;
-            else if (fix[c] == 2) { lw[1] += T(2) * lv; lB[bl] -= lv; }
-            else { lw[1] += lv; slope_vjp(sw[c], th, sgn * lv, lw[0], lw[1], lw[2]); }
+            else { lw[1] += T(2) * lv; lB[bl] -= lv; }
         } else {
             if (fix[c] == 1) { lw[2] += T(2) * lv; lB[bh] -= lv; }
-            else if (fix[c] == 2) lB[bl] += lv;
-            else { lw[2] += lv; slope_vjp(sw[c], th, sgn * lv, lw[1], lw[2], lw[3]); }
+            else lB[bl] += lv;
         }
         lP[c + 1] += lf[c][1];
-        slope_vjp(sP[c], th, sgn * lf[c][1], lP[c], lP[c + 1], lP[c + 2]);
+        slope_vjp(sP[c], th2, q4 * lf[c][1], lP[c], lP[c + 1], lP[c + 2]);
         lQ[c + 1] += lf[c][2];
-        slope_vjp(sQ[c], th, sgn * lf[c][2], lQ[c], lQ[c + 1], lQ[c + 2]);
+        slope_vjp(sQ[c], th2, q4 * lf[c][2], lQ[c], lQ[c + 1], lQ[c + 2]);
     }
 }
 
@@ -400,29 +421,32 @@ __device__ __forceinline__ size_t corner_index(const Geo &G, int ci, int cj)
     return (size_t)(cj + 1) * G.pc + (ci + 1);
 }
 
+// The mask and history passes' tiles: 32 columns by 8 rows, a cell per thread
+// (200 x 150 FP64 cells: 133 blocks where 32 x 32 tiles gave 35).
+constexpr int kEX = 32, kEY = 8;
+
 // Step 1 of the reverse: the masks; the state's own path (w^{n+1} = w^n +
-// ...) passes the masked adjoint on unchanged.  One 32 x 32 tile per block
-// of 32 x 32 threads, a cell per thread; the y-lines' right side
+// ...) passes the masked adjoint on unchanged.  The y-lines' right side
 // (column-major) is transposed in shared memory and written along columns.
 template <typename real>
-__global__ void __launch_bounds__(1024) k_adj_mask(AdjArgs<real> A)
+__global__ void __launch_bounds__(kEX * kEY) k_adj_mask(const __grid_constant__ AdjArgs<real> A)
 {
     dependent_launch_wait_then_release();
-    __shared__ real tq[32][33];
+    __shared__ real tq[kEY][kEX + 1];
     const Geo &G = A.geo;
-    const int tx = threadIdx.x, ty = threadIdx.y, bx = blockIdx.x * 32, by = blockIdx.y * 32;
+    const int tx = threadIdx.x, ty = threadIdx.y, bx = blockIdx.x * kEX, by = blockIdx.y * kEY;
     const int i = bx + tx, j = by + ty;
     real lq = real(0);
     if (i < G.nx && j < G.ny) {
         const int k = j * G.nx + i;
         const real Bb = bbar_at(A.Bc, G, i, j);
         const real ws = A.c.ws;
-        const real d = fmax(ws - Bb, real(0));
         const real gam = A.final_stage ? sponge_gamma<real>(A.c, G, i, j) : real(1);
         const real wn = A.w_next[k];
         const bool dry = wn - Bb <= real(0);
-        const bool spw = gam < real(1) && d > real(0);
-        const real w1 = spw ? ws + (wn - ws) / gam : wn;   // before the sponge
+        const bool spw = gam < real(1) && ws > Bb;
+        real w1 = wn;   // before the sponge
+        if (spw) w1 = ws + (wn - ws) / gam;
         const real tol = (sizeof(real) == 8 ? real(1e-12) : real(1e-6)) * fmax(real(1), fabs(Bb));
         const bool clamped = w1 - Bb <= tol;
         if (clamped && A.lBb) A.lBb[ring_index(G, i, j)] += A.lw[k] * (spw ? gam : real(1));   // w = Bbar there
@@ -437,33 +461,32 @@ __global__ void __launch_bounds__(1024) k_adj_mask(AdjArgs<real> A)
     if (A.packX) {
         tq[ty][tx] = lq;
         __syncthreads();
-        const int ic = bx + ty, jc = by + tx;
-        if (ic < G.nx && jc < G.ny) A.packY[(size_t)ic * G.py + jc] = tq[tx][ty];
+        const int t = ty * kEX + tx, c = t / kEY, r = t % kEY;
+        if (bx + c < G.nx && by + r < G.ny) A.packY[(size_t)(bx + c) * G.py + by + r] = tq[r][c];
     }
 }
 
 // Step 3: the history.  The increments of w, U* and V* weigh R^n, R^{n-1},
 // R^{n-2} by c0, c1, c2 and (U*, V*) the mixed terms F*, G* by e0, e1, e2.
-// One 32 x 32 tile per block of 32 x 32 threads, a cell per thread; the
-// y-lines' solution (column-major) is read along its columns and transposed
+// A cell per thread; the y-lines' solution (column-major) is read along its columns and transposed
 // in shared memory.
 template <typename real>
-__global__ void __launch_bounds__(1024) k_adj_hist(AdjArgs<real> A)
+__global__ void __launch_bounds__(kEX * kEY) k_adj_hist(const __grid_constant__ AdjArgs<real> A)
 {
     dependent_launch_wait_then_release();
-    __shared__ real tq[32][33];
+    __shared__ real tq[kEY][kEX + 1];
     const Geo &G = A.geo;
-    const int tx = threadIdx.x, ty = threadIdx.y, bx = blockIdx.x * 32, by = blockIdx.y * 32;
+    const int tx = threadIdx.x, ty = threadIdx.y, bx = blockIdx.x * kEX, by = blockIdx.y * kEY;
     if (A.muY) {
-        const int i = bx + ty, j = by + tx;
-        tq[ty][tx] = i < G.nx && j < G.ny ? A.muY[(size_t)i * G.py + j] : real(0);
+        const int t = ty * kEX + tx, c = t / kEY, r = t % kEY;
+        tq[r][c] = bx + c < G.nx && by + r < G.ny ? A.muY[(size_t)(bx + c) * G.py + by + r] : real(0);
         __syncthreads();
     }
     const int i = bx + tx, j = by + ty;
     if (i >= G.nx || j >= G.ny) return;
     const int k = j * G.nx + i;
     const real mu = A.muX ? A.muX[(size_t)j * G.px + i] : A.ldU[k];
-    const real mv = A.muY ? tq[tx][ty] : A.ldV[k];
+    const real mv = A.muY ? tq[ty][tx] : A.ldV[k];
     const real m[5] = {A.lw[k], mu, mv, mu, mv};
 #pragma unroll
     for (int v = 0; v < 5; v++) {
@@ -504,21 +527,30 @@ __device__ __forceinline__ void cell_vjp(const AdjArgs<real> &A, int i, int j, c
         // derivative 0 at 0)
         const real P0 = acc.val(i, j, 1), Q0 = acc.val(i, j, 2);
         const real hb = acc.val(i, j, 0) - Bb;
-        const bool hpos = hb >= real(0);
-        const real hp = hpos ? hb : real(0);
-        const real hinv = desing(hp, A.c.eps);
         const bool man = A.phy.friction == kFricManning;
-        const real cr = man ? cel::cbrt_r(hinv) : real(1);
-        const real fc = man ? A.c.fric * cr : A.c.fric;
-        const real dfc = man && hinv > real(0) ? A.c.fric / (real(3) * cr * cr) : real(0);
-        const real mag = sqrt(P0 * P0 + Q0 * Q0);
-        const real Aq = lF * P0 + lG * Q0;
-        const real k2 = hinv * hinv;
-        dfw = hpos ? -mag * Aq * (dfc * k2 + real(2) * fc * hinv) * desing_dh(hp, A.c.eps) : real(0);
-        const real um = mag > real(0) ? Aq / mag : real(0);
+        const real m2 = P0 * P0 + Q0 * Q0;
+        const real mag = sqrt_r(m2), Aq = lF * P0 + lG * Q0;
+        const real um = mag > real(0) ? Aq * rcp_r(mag) : real(0);
+        real fk;   // fc k^2, and -d(fc k^2)/dh in gk
+        real gk;
+        if (at_least(hb, A.c.hwet)) {   // k = 1/h: f h^-2, or f h^(-7/3)
+            const real k1 = rcp_r(hb);
+            fk = friction_depth(A.phy.friction, A.c.fric, hb, A.c.eps, A.c.hwet);
+            gk = (man ? real(7.0 / 3.0) : real(2)) * fk * k1;
+        } else {
+            const bool hpos = hb >= real(0);
+            const real hp = hpos ? hb : real(0);
+            const real hinv = desing(hp, A.c.eps);
+            const real cr = man ? cel::cbrt_r(hinv) : real(1);
+            const real fc = man ? A.c.fric * cr : A.c.fric;
+            const real dfc = man && hinv > real(0) ? A.c.fric / (real(3) * cr * cr) : real(0);
+            fk = fc * (hinv * hinv);
+            gk = hpos ? -(dfc * (hinv * hinv) + real(2) * fc * hinv) * desing_dh(hp, A.c.eps) : real(0);
+        }
+        dfw = mag * Aq * gk;
         dw += dfw;
-        dP = -fc * k2 * (P0 * um + mag * lF);
-        dQ = -fc * k2 * (Q0 * um + mag * lG);
+        dP = -fk * (P0 * um + mag * lF);
+        dQ = -fk * (Q0 * um + mag * lG);
     }
     if (A.lBc) {   // the bed: Bbar through h = w - Bbar, the face beds through the slope
         const real hb = acc.val(i, j, 0) - Bb;
@@ -571,7 +603,7 @@ __device__ __forceinline__ void face_vjp(const AdjArgs<real> &A, int dir, int f,
         P[q] = acc.val(i, j, 1);
         Q[q] = acc.val(i, j, 2);
     }
-    face_flux_vjp(w, P, Q, Bm, Bf, Bp, A.c.theta, A.c.g, A.c.eps, dir, lH, lw, lP, lQ, lB);
+    face_flux_vjp(w, P, Q, Bm, Bf, Bp, A.c.th2, A.c.g, A.c.eps, A.c.hwet, dir, lH, lw, lP, lQ, lB);
 #pragma unroll
     for (int c = 0; c < 4; c++) {
         int i, j;
@@ -616,7 +648,8 @@ __global__ void k_face_vjp_check(const real *in, int n, real *out)
     const int dir = x[21] != real(0) ? 1 : 0;
     face_flux_vjp_dual(x, x + 4, x + 8, x[12], x[13], x[14], x[18], x[19], x[20], dir, x + 15, o);
     real lw[4] = {0, 0, 0, 0}, lP[4] = {0, 0, 0, 0}, lQ[4] = {0, 0, 0, 0}, lB[3] = {0, 0, 0};
-    face_flux_vjp(x, x + 4, x + 8, x[12], x[13], x[14], x[18], x[19], x[20], dir, x + 15, lw, lP, lQ, lB);
+    face_flux_vjp(x, x + 4, x + 8, x[12], x[13], x[14], real(2) * x[18], x[19], x[20], sqrt(sqrt(x[20])), dir, x + 15, lw, lP,
+                  lQ, lB);
     for (int q = 0; q < 4; q++) {
         o[15 + q] = lw[q];
         o[19 + q] = lP[q];
@@ -666,7 +699,6 @@ __device__ __forceinline__ void disp_vjp(const AdjArgs<real> &A, int i, int j, c
         {-1, -1, axy - bxyy - bxxy}};
 #pragma unroll
     for (int q = 0; q < 13; q++) {
-        if (pts[q].wgt == real(0)) continue;
         const Src<real> s = acc.map(i + pts[q].di, j + pts[q].dj);
         if (s.idx >= 0) acc.cell(0, s.ci, s.cj, pts[q].wgt);
         else acc.ghost(s, 0, pts[q].wgt);
@@ -792,21 +824,18 @@ struct TileAcc : TileData<real> {
     }
     __device__ __forceinline__ void cell(int var, int i, int j, real v) const
     {
-        if (v == real(0)) return;
         const int li = i - D::x0 + 2, lj = j - D::y0 + 2;
         if (kInt || (li >= 0 && li < kVW && lj >= 0 && lj < kWH)) atomicAdd(D::sv[var] + lj * kVWS + li, v);
         else atomicAdd(D::gv[var] + (size_t)j * D::nx + i, v);
     }
     __device__ __forceinline__ void ring(int i, int j, real v) const
     {
-        if (v == real(0)) return;
         const int li = i - D::x0 + 2, lj = j - D::y0 + 2;
         if (kInt || (li >= 0 && li < kVW && lj >= 0 && lj < kWH)) atomicAdd(D::sd + lj * kVWS + li, v);
         else atomicAdd(D::gd + (size_t)(j + 1) * (D::nx + 2) + (i + 1), v);
     }
     __device__ __forceinline__ void corner(int ci, int cj, real v) const
     {
-        if (v == real(0)) return;
         const int li = ci - D::x0 + 2, lj = cj - D::y0 + 2;
         if (kInt || (li >= 0 && li < kVC && lj >= 0 && lj < kCH)) atomicAdd(D::sc + lj * kVCS + li, v);
         else atomicAdd(D::gc + (size_t)(cj + 1) * D::pc + (ci + 1), v);
@@ -1098,7 +1127,7 @@ __global__ void k_adj_misfit(AdjArgs<real> A, const int32_t *gij, int ng, const 
 template <typename real>
 cudaError_t launch_adjoint_mask(const AdjArgs<real> &a, cudaStream_t st)
 {
-    dim3 b(32, 32), g((a.geo.nx + 31) / 32, (a.geo.ny + 31) / 32);
+    dim3 b(kEX, kEY), g((a.geo.nx + kEX - 1) / kEX, (a.geo.ny + kEY - 1) / kEY);
     cudaError_t e = launch_step_kernel(k_adj_mask<real>, g, b, 0, st, a);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -1106,7 +1135,7 @@ cudaError_t launch_adjoint_mask(const AdjArgs<real> &a, cudaStream_t st)
 template <typename real>
 cudaError_t launch_adjoint_hist(const AdjArgs<real> &a, cudaStream_t st)
 {
-    dim3 b(32, 32), g((a.geo.nx + 31) / 32, (a.geo.ny + 31) / 32);
+    dim3 b(kEX, kEY), g((a.geo.nx + kEX - 1) / kEX, (a.geo.ny + kEY - 1) / kEY);
     cudaError_t e = launch_step_kernel(k_adj_hist<real>, g, b, 0, st, a);
     return e != cudaSuccess ? e : cudaGetLastError();
 }

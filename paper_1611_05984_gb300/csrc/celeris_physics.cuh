@@ -144,6 +144,9 @@ __device__ __forceinline__ double sqrt_r(double x)
     return __double_as_longlong(x) == 0 ? 0.0 : sqrt(x);
 }
 
+// 1 / sqrt(x)
+__device__ __forceinline__ float rsqrt_r(float x) { return rsqrtf(x); }
+
 // sqrt(x) and c / x' for x = g h, c = g: the celerity and 1/h from one root.
 __device__ __forceinline__ void root_and_inverse(float g, float h, float gh, float &s, float &ih)
 {
@@ -229,6 +232,45 @@ __device__ __forceinline__ double minmod_r(double a, double b, double c)
     const unsigned long long kc = (unsigned long long)__double_as_longlong(c);
     const unsigned long long ac = ka < kc ? ka : kc, m = ac < kb ? ac : kb;
     return (long long)(ka ^ kc) < 0 ? 0.0 : __longlong_as_double((long long)m);
+}
+
+// The same with the choice kept: 1, 2 or 3 for a, b or c, 0 for none (ties to
+// a, then to b).
+__device__ __forceinline__ int minmod_choice(float a, float b, float c, float &m)
+{
+    const bool b_c = fabsf(b) <= fabsf(c);
+    const float mbc = b_c ? b : c;
+    const bool first = fabsf(a) <= fabsf(mbc);
+    m = first ? a : mbc;
+    int s = first ? 1 : (b_c ? 2 : 3);
+    if ((__float_as_int(a) ^ __float_as_int(c)) < 0 || m == 0.f) {
+        s = 0;
+        m = 0.f;
+    }
+    return s;
+}
+__device__ __forceinline__ int minmod_choice(double a, double b, double c, double &m)
+{
+    const unsigned long long ka = (unsigned long long)__double_as_longlong(a);
+    const unsigned long long kb = (unsigned long long)__double_as_longlong(b);
+    const unsigned long long kc = (unsigned long long)__double_as_longlong(c);
+    const bool b_c = kb <= kc;
+    const unsigned long long kbc = b_c ? kb : kc, k = ka <= kbc ? ka : kbc;
+    int s = ka <= kbc ? 1 : (b_c ? 2 : 3);
+    if ((long long)(ka ^ kc) < 0 || (k << 1) == 0ull) s = 0;
+    m = s ? __longlong_as_double((long long)k) : 0.0;
+    return s;
+}
+
+// x >= 0 (false for NaN) and a >= b (FP64: as integers; for finite values)
+__device__ __forceinline__ bool not_below(float x) { return x >= 0.f; }
+__device__ __forceinline__ bool not_below(double x) { return __double2hiint(x) >= 0 || (__double_as_longlong(x) << 1) == 0; }
+__device__ __forceinline__ bool ge_r(float a, float b) { return a >= b; }
+__device__ __forceinline__ bool ge_r(double a, double b)
+{
+    // -0 and 0 are equal
+    const long long ka = order_key(a), kb = order_key(b);
+    return ka >= kb || ((__double_as_longlong(a) | __double_as_longlong(b)) << 1) == 0;
 }
 
 // One cell's reconstruction along a direction, cells fed in order: q the
