@@ -431,7 +431,7 @@ constexpr int kEX = 32, kEY = 8;
 template <typename real>
 __global__ void __launch_bounds__(kEX * kEY) k_adj_mask(const __grid_constant__ AdjArgs<real> A)
 {
-    dependent_launch_wait_then_release();
+    dependent_launch_wait();
     __shared__ real tq[kEY][kEX + 1];
     const Geo &G = A.geo;
     const int tx = threadIdx.x, ty = threadIdx.y, bx = blockIdx.x * kEX, by = blockIdx.y * kEY;
@@ -464,6 +464,7 @@ __global__ void __launch_bounds__(kEX * kEY) k_adj_mask(const __grid_constant__ 
         const int t = ty * kEX + tx, c = t / kEY, r = t % kEY;
         if (bx + c < G.nx && by + r < G.ny) A.packY[(size_t)(bx + c) * G.py + by + r] = tq[r][c];
     }
+    dependent_launch_release();
 }
 
 // Step 3: the history.  The increments of w, U* and V* weigh R^n, R^{n-1},
@@ -473,7 +474,7 @@ __global__ void __launch_bounds__(kEX * kEY) k_adj_mask(const __grid_constant__ 
 template <typename real>
 __global__ void __launch_bounds__(kEX * kEY) k_adj_hist(const __grid_constant__ AdjArgs<real> A)
 {
-    dependent_launch_wait_then_release();
+    dependent_launch_wait();
     __shared__ real tq[kEY][kEX + 1];
     const Geo &G = A.geo;
     const int tx = threadIdx.x, ty = threadIdx.y, bx = blockIdx.x * kEX, by = blockIdx.y * kEY;
@@ -483,7 +484,10 @@ __global__ void __launch_bounds__(kEX * kEY) k_adj_hist(const __grid_constant__ 
         __syncthreads();
     }
     const int i = bx + tx, j = by + ty;
-    if (i >= G.nx || j >= G.ny) return;
+    if (i >= G.nx || j >= G.ny) {
+        dependent_launch_release();
+        return;
+    }
     const int k = j * G.nx + i;
     const real mu = A.muX ? A.muX[(size_t)j * G.px + i] : A.ldU[k];
     const real mv = A.muY ? tq[ty][tx] : A.ldV[k];
@@ -502,6 +506,7 @@ __global__ void __launch_bounds__(kEX * kEY) k_adj_hist(const __grid_constant__ 
         A.accP[k] += A.lP[k];
         A.accQ[k] += A.lQ[k];
     }
+    dependent_launch_release();
 }
 
 // Bed slope and friction (Eq. 9-10, 31-32) at cell (i, j): no neighbours.
@@ -767,7 +772,7 @@ constexpr int kVW = kVT + 4;         // cell window: x0 - 2 .. x0 + 33
 constexpr int kVWS = kVW + 1;
 constexpr int kVC = kVT + 5;         // corner window: x0 - 2 .. x0 + 34
 constexpr int kVCS = kVC + 1;
-constexpr int kVjpThreads = 256;
+constexpr int kVjpThreads = 256;     // 512 where a block has its SM to itself (launch_vjp_rows)
 
 // The accumulator's pointers and tile position.
 template <typename real>
@@ -842,8 +847,9 @@ struct TileAcc : TileData<real> {
     }
 };
 
-// The tile's cells and faces.
-template <typename real, int TY, bool kInt>
+// The tile's cells and faces: a warp takes rows of cells, of x-faces and of
+// y-faces in turn (NT threads).
+template <typename real, int TY, int NT, bool kInt>
 __device__ __forceinline__ void vjp_tile_work(const AdjArgs<real> &A, const TileData<real> &td, int tx, int ty)
 {
     TileAcc<real, TY, kInt> acc;
@@ -851,7 +857,26 @@ __device__ __forceinline__ void vjp_tile_work(const AdjArgs<real> &A, const Tile
     const Geo &G = A.geo;
     const int x0 = td.x0, y0 = td.y0;
     const int xe = min(x0 + kVT, G.nx), ye = min(y0 + TY, G.ny);
-    for (int j = y0 + ty; j < ye; j += kVjpThreads / 32) {
+    if constexpr (NT / 32 > TY) {   // more warps than rows: the three kinds side by side
+        const int nr = ye - y0, ng = nr + (ye == G.ny ? 1 : 0);
+        for (int t = ty; t < 2 * nr + ng; t += NT / 32) {
+            if (t < nr) {
+                const int i = x0 + tx, j = y0 + t;
+                if (i < xe) {
+                    cell_vjp(A, i, j, acc);
+                    if (A.bsnq) disp_vjp(A, i, j, acc);
+                }
+            } else if (t < 2 * nr) {
+                const int fe = xe + (xe == G.nx ? 1 : 0);
+                for (int f = x0 + tx; f < fe; f += 32) face_vjp(A, 0, f, y0 + t - nr, acc);
+            } else {
+                const int i = x0 + tx;
+                if (i < xe) face_vjp(A, 1, y0 + t - 2 * nr, i, acc);
+            }
+        }
+        return;
+    }
+    for (int j = y0 + ty; j < ye; j += NT / 32) {
         const int i = x0 + tx;
         if (i < xe) {
             cell_vjp(A, i, j, acc);
@@ -859,10 +884,10 @@ __device__ __forceinline__ void vjp_tile_work(const AdjArgs<real> &A, const Tile
         }
     }
     const int fe = xe + (xe == G.nx ? 1 : 0);
-    for (int j = y0 + ty; j < ye; j += kVjpThreads / 32)
+    for (int j = y0 + ty; j < ye; j += NT / 32)
         for (int f = x0 + tx; f < fe; f += 32) face_vjp(A, 0, f, j, acc);
     const int ge = ye + (ye == G.ny ? 1 : 0);
-    for (int gq = y0 + ty; gq < ge; gq += kVjpThreads / 32) {
+    for (int gq = y0 + ty; gq < ge; gq += NT / 32) {
         const int i = x0 + tx;
         if (i < xe) face_vjp(A, 1, gq, i, acc);
     }
@@ -874,10 +899,10 @@ constexpr size_t vjp_smem_bytes()
     return sizeof(real) * (size_t)(7 * (TY + 4) * kVWS + 2 * (TY + 5) * kVCS);
 }
 
-template <typename real, int TY>
-__global__ void __launch_bounds__(kVjpThreads, sizeof(real) == 4 ? 4 : 2) k_adj_vjp(const __grid_constant__ AdjArgs<real> A)
+template <typename real, int TY, int NT>
+__global__ void __launch_bounds__(NT, NT > 256 ? 1 : (sizeof(real) == 4 ? 4 : 2)) k_adj_vjp(const __grid_constant__ AdjArgs<real> A)
 {
-    dependent_launch_wait_then_release();
+    dependent_launch_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     real *sm = reinterpret_cast<real *>(smem_raw);
     const Geo &G = A.geo;
@@ -885,7 +910,7 @@ __global__ void __launch_bounds__(kVjpThreads, sizeof(real) == 4 ? 4 : 2) k_adj_
     const int x0 = blockIdx.x * kVT, y0 = blockIdx.y * TY;
     const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
     constexpr int ntot = 4 * kWH * kVWS + kCH * kVCS;
-    for (int k = tid; k < ntot; k += kVjpThreads) sm[k] = real(0);
+    for (int k = tid; k < ntot; k += NT) sm[k] = real(0);
     TileData<real> acc;
     for (int v = 0; v < 3; v++) acc.sv[v] = sm + v * kWH * kVWS;
     acc.sd = sm + 3 * kWH * kVWS;
@@ -902,14 +927,14 @@ __global__ void __launch_bounds__(kVjpThreads, sizeof(real) == 4 ? 4 : 2) k_adj_
     acc.npos = A.c.npos;
     // the state with its ghosts (source2d) on cells within 2 of the grid,
     // and the bed corners, over the windows
-    for (int k = tid; k < kVW * kWH; k += kVjpThreads) {
+    for (int k = tid; k < kVW * kWH; k += NT) {
         const int li = k % kVW, lj = k / kVW, i = x0 - 2 + li, j = y0 - 2 + lj, o = lj * kVWS + li;
         if (i >= -2 && i <= G.nx + 1 && j >= -2 && j <= G.ny + 1) {
             const Src<real> q = source2d(A, i, j);
             for (int v = 0; v < 3; v++) xs[v * kWH * kVWS + o] = q.v[v];
         }
     }
-    for (int k = tid; k < kVC * kCH; k += kVjpThreads) {
+    for (int k = tid; k < kVC * kCH; k += NT) {
         const int li = k % kVC, lj = k / kVC, ci = x0 - 2 + li, cj = y0 - 2 + lj;
         if (ci >= -1 && ci <= G.nx + 1 && cj >= -1 && cj <= G.ny + 1) xb[lj * kVCS + li] = corner(A.Bc, G, ci, cj);
     }
@@ -923,10 +948,11 @@ __global__ void __launch_bounds__(kVjpThreads, sizeof(real) == 4 ? 4 : 2) k_adj_
     acc.nx = G.nx;
     acc.pc = G.pc;
     __syncthreads();
-    if (acc.interior) vjp_tile_work<real, TY, true>(A, acc, tx, ty);
-    else vjp_tile_work<real, TY, false>(A, acc, tx, ty);
+    if (acc.interior) vjp_tile_work<real, TY, NT, true>(A, acc, tx, ty);
+    else vjp_tile_work<real, TY, NT, false>(A, acc, tx, ty);
     __syncthreads();
-    for (int k = tid; k < kVW * kWH; k += kVjpThreads) {
+    dependent_launch_release();
+    for (int k = tid; k < kVW * kWH; k += NT) {
         const int li = k % kVW, lj = k / kVW, i = x0 - 2 + li, j = y0 - 2 + lj, o = lj * kVWS + li;
         if (i >= 0 && i < G.nx && j >= 0 && j < G.ny) {
             const size_t c = (size_t)j * G.nx + i;
@@ -937,7 +963,7 @@ __global__ void __launch_bounds__(kVjpThreads, sizeof(real) == 4 ? 4 : 2) k_adj_
             atomicAdd(A.ld + ring_index(G, i, j), acc.sd[o]);
     }
     if (A.lBc)
-        for (int k = tid; k < kVC * kCH; k += kVjpThreads) {
+        for (int k = tid; k < kVC * kCH; k += NT) {
             const int li = k % kVC, lj = k / kVC, ci = x0 - 2 + li, cj = y0 - 2 + lj;
             const real v = acc.sc[lj * kVCS + li];
             if (v != real(0) && ci >= -1 && ci <= G.nx + 1 && cj >= -1 && cj <= G.ny + 1)
@@ -1140,24 +1166,7 @@ cudaError_t launch_adjoint_hist(const AdjArgs<real> &a, cudaStream_t st)
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-template <typename real, int TY>
-cudaError_t launch_vjp_rows(const AdjArgs<real> &a, cudaStream_t st)
-{
-    constexpr size_t smem = vjp_smem_bytes<real, TY>();
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(k_adj_vjp<real, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
-    dim3 g((a.geo.nx + kVT - 1) / kVT, (a.geo.ny + TY - 1) / TY);
-    cudaError_t e = launch_step_kernel(k_adj_vjp<real, TY>, g, dim3(kVjpThreads), smem, st, a);
-    return e != cudaSuccess ? e : cudaGetLastError();
-}
-
-// Tile rows of the Jacobian kernel: 32 while 32 x 32 tiles give every SM
-// several blocks, else 16 or 8, so that small grids still fill the GPU.
-static int vjp_tile_rows(int nx, int ny)
+static int sm_count()
 {
     static int nsm = 0;
     if (nsm == 0) {
@@ -1165,7 +1174,32 @@ static int vjp_tile_rows(int nx, int ny)
         if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             nsm = 1;
     }
-    const long cols = (nx + kVT - 1) / kVT, want = 4L * nsm;
+    return nsm;
+}
+
+template <typename real, int TY, int NT>
+cudaError_t launch_vjp_rows(const AdjArgs<real> &a, cudaStream_t st)
+{
+    // 512 threads: a block to an SM, which the shared memory asked for sees to
+    constexpr size_t smem = NT > 256 ? (size_t)120 * 1024 : vjp_smem_bytes<real, TY>();
+    static_assert(smem >= vjp_smem_bytes<real, TY>(), "the tile's windows");
+    static bool configured = false;
+    if (!configured) {
+        cudaError_t e =
+            cudaFuncSetAttribute(k_adj_vjp<real, TY, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        configured = true;
+    }
+    dim3 g((a.geo.nx + kVT - 1) / kVT, (a.geo.ny + TY - 1) / TY);
+    cudaError_t e = launch_step_kernel(k_adj_vjp<real, TY, NT>, g, dim3(NT), smem, st, a);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+// Tile rows of the Jacobian kernel: 32 while 32 x 32 tiles give every SM
+// several blocks, else 16 or 8, so that small grids still fill the GPU.
+static int vjp_tile_rows(int nx, int ny)
+{
+    const long cols = (nx + kVT - 1) / kVT, want = 4L * sm_count();
     if (cols * ((ny + 31) / 32) >= want) return 32;
     if (cols * ((ny + 15) / 16) >= want) return 16;
     return 8;
@@ -1175,10 +1209,15 @@ template <typename real>
 cudaError_t launch_adjoint_vjp(const AdjArgs<real> &a, cudaStream_t st)
 {
     switch (vjp_tile_rows(a.geo.nx, a.geo.ny)) {
-    case 32: return launch_vjp_rows<real, 32>(a, st);
-    case 16: return launch_vjp_rows<real, 16>(a, st);
-    default: return launch_vjp_rows<real, 8>(a, st);
+    case 32: return launch_vjp_rows<real, 32, kVjpThreads>(a, st);
+    case 16: return launch_vjp_rows<real, 16, kVjpThreads>(a, st);
+    default: break;
     }
+    // FP64 (bound by each SM's own FP64 pipe) on a grid of no more tiles than
+    // SMs: one block per SM, with twice the warps
+    const long blocks = (long)((a.geo.nx + kVT - 1) / kVT) * ((a.geo.ny + 7) / 8);
+    if (sizeof(real) == 8 && blocks <= sm_count()) return launch_vjp_rows<real, 8, 512>(a, st);
+    return launch_vjp_rows<real, 8, kVjpThreads>(a, st);
 }
 
 template <typename real>

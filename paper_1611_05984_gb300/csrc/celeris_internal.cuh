@@ -326,14 +326,32 @@ int dependent_launch();
 // A kernel launched with programmatic stream serialisation may start while
 // the kernel before it on the stream drains its last blocks.  Each such
 // kernel first waits for that kernel to complete (its writes visible),
-// before any access to memory, then lets the kernel after it launch: the
-// kernels overlap only in their launch and block scheduling, never in their
-// memory accesses.  Without the launch attribute the wait returns at once.
-__device__ __forceinline__ void dependent_launch_wait_then_release()
+// before any access to memory that kernel writes; the kernels overlap only in
+// their launch and block scheduling, never in those accesses.  Without the
+// launch attribute the wait returns at once.
+//
+// A kernel lets the one after it launch (release) when its blocks are done,
+// not when they start: blocks that start early take their places beside the
+// ones still running, so a compute-bound grid of about one block per SM ends
+// up with two on some SMs and none on others (FP64 gradient of 200 x 150
+// cells, with its Jacobian kernel held to one block per SM as well: 14.4 ms a
+// pass with the release at the start, 10.0 at the end; 601 x 601 FP32 island
+// 838 -> 792 us, 2048 x 2048 beach 4181 -> 4132 us).  Only a grid that leaves
+// most SMs free lets the next kernel start at once (559 x 4 beach 722 us, 733
+// with the release at the end).
+__device__ __forceinline__ void dependent_launch_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dependent_launch_release()
 {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+// For the short kernels, whose own blocks are quickly gone.
+__device__ __forceinline__ void dependent_launch_wait_then_release()
+{
+    dependent_launch_wait();
+    dependent_launch_release();
+}
+// The stencils' release at their start: a grid of few blocks.
+__device__ __forceinline__ bool releases_early() { return gridDim.x * gridDim.y <= 64; }
 
 // A step kernel's launch, with programmatic stream serialisation where it is
 // switched on (the kernel's own wait keeps its memory accesses after the

@@ -899,8 +899,10 @@ template <int kSpec, int TY>
 __global__ void __launch_bounds__(kStencilThreads, 2) k_stencil(const __grid_constant__ StencilArgs<double> A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    dependent_launch_wait_then_release();
+    dependent_launch_wait();
+    if (releases_early()) dependent_launch_release();
     stencil_tile<double, kSpec, TY>(A, GridOrigin<TY>(), smem_raw);
+    if (!releases_early()) dependent_launch_release();
 }
 
 // FP32 (celeris_stencil_f32.cuh): 64 columns and 4 kR rows per block.
@@ -920,9 +922,11 @@ template <int kSpec, int kR>
 __global__ void __launch_bounds__(kPThreads, 4) k_stencil_pair(const __grid_constant__ StencilArgs<float> A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    dependent_launch_wait_then_release();
+    dependent_launch_wait();
+    if (releases_early()) dependent_launch_release();
     stencil_tile_pair<kSpec, kR>(A, blockIdx.x * kPW, blockIdx.y * PairSmem<kR>::TH, smem_raw, threadIdx.x,
                                  BlockBarrier());
+    if (!releases_early()) dependent_launch_release();
 }
 
 // Copy a scenario's argument block (device memory) into shared memory.
@@ -1184,7 +1188,7 @@ __device__ __forceinline__ void line_solve_reg(const LineArgs<real> &A, int line
     }
     real r[M];
     auto load_rhs = [&]() {
-        dependent_launch_wait_then_release();
+        dependent_launch_wait();
         if (any) {
             if (kMode == 0)   // the dry bits, read in the epilogue
                 asm volatile("prefetch.global.L1 [%0];" ::"l"(A.mask + (size_t)line * A.nwords + (f >> 5)));
@@ -1760,6 +1764,7 @@ __global__ void __launch_bounds__(kOcc ? 256 : (sizeof(real) == 4 ? 1024 : 512),
     const int fam = blockIdx.x < PA.L[0].nlines ? 0 : 1;
     const int line = fam == 0 ? blockIdx.x : blockIdx.x - PA.L[0].nlines;
     line_solve_any<real, kMode>(PA.L[fam], line, L);
+    dependent_launch_release();
 }
 
 template <typename real, int M, int kMode>
