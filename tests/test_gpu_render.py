@@ -71,3 +71,20 @@ def test_render_rejects_bad_parameters():
                dict(grid=-1.0), dict(zmin=2.0, zmax=1.0)):
         with pytest.raises(celeris.CelerisError):
             g.render(celeris.render_params(**kw))
+
+
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+@pytest.mark.parametrize("nx,ny", [(2, 2), (31, 33), (32, 32), (33, 64), (97, 31)])
+def test_render_tile_edges(oracle_mod, prec, nx, ny):
+    """One pixel short of, at and past the 32 x 32 tiles, every mode, byte for
+    byte; the bed rises above the water on the way."""
+    from paper_1611_05984_gb300 import celeris
+    s = sc.beach(nx=nx, ny=ny, dx=430.0 / nx, sponge=1)
+    x, y = np.arange(nx) / nx, np.arange(ny) / ny
+    s.w0 = np.maximum(s.z, 0.3 * np.sin(9.0 * x)[None, :] * np.cos(5.0 * y)[:, None])
+    s.P0 = np.where(s.z < -0.5, s.w0, 0.0)
+    s.Q0 = 0.4 * s.P0
+    g = celeris.from_scenario(s, dtype=torch.float64 if prec == "f64" else torch.float32)
+    for kw in CASES:
+        img = g.render(celeris.render_params(**kw)).cpu().numpy()
+        np.testing.assert_array_equal(img, _oracle_image(oracle_mod, s, g, kw))
