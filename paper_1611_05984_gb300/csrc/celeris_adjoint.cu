@@ -1215,8 +1215,10 @@ cudaError_t launch_adjoint_vjp(const AdjArgs<real> &a, cudaStream_t st)
     }
     // FP64 (bound by each SM's own FP64 pipe) on a grid of no more tiles than
     // SMs: one block per SM, with twice the warps
-    const long blocks = (long)((a.geo.nx + kVT - 1) / kVT) * ((a.geo.ny + 7) / 8);
-    if (sizeof(real) == 8 && blocks <= sm_count()) return launch_vjp_rows<real, 8, 512>(a, st);
+    if constexpr (sizeof(real) == 8) {
+        const long blocks = (long)((a.geo.nx + kVT - 1) / kVT) * ((a.geo.ny + 7) / 8);
+        if (blocks <= sm_count()) return launch_vjp_rows<real, 8, 512>(a, st);
+    }
     return launch_vjp_rows<real, 8, kVjpThreads>(a, st);
 }
 
