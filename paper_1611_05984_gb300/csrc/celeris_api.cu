@@ -355,8 +355,6 @@ LineArgs<real> line_args(const cel_solver *s, const Coef<real> &coef, int dir, i
     l.rh2 = real(1.0 / (h * h));
     l.hrh = real(0.5 / h);
     l.srh = real(1.0 / (6.0 * h));
-    l.kr = real((s->phy.Bd + 1.0 / 3.0) / (h * h));
-    l.ks = real(1.0 / (12.0 * h * h));
     l.rhs = s->at<real>(dir == 0 ? L.U : L.Vc);
     l.d = s->at<real>(dir == 0 ? L.dr : L.dc);
     l.mask = s->at<uint32_t>(dir == 0 ? L.mr : L.mc);

@@ -231,7 +231,6 @@ struct LineArgs {
     int final_stage;       // apply the sponge
     int identity;          // NLSW model: no dispersive solve, P = U*, Q = V*
     real rh, rh2, hrh, srh; // 1/h, 1/h^2, 1/(2h), 1/(6h) along the line
-    real kr, ks;            // (B + 1/3) / h^2 and 1/(12 h^2) (the register path's rows)
 };
 
 // Headless rendering of the state (celeris_render.cu).

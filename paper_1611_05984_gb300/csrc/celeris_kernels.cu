@@ -987,16 +987,6 @@ __device__ __forceinline__ void coef23(real B3, real hrh, real srh, real rh2, re
     c = -s - r;
 }
 
-// The same from the constants folded per line (register path).
-template <typename real>
-__device__ __forceinline__ void coef23_folded(real kr, real ks, real dd, real dm, real dp, real &a, real &b, real &c)
-{
-    const real r = (dd * dd) * kr, s = (dd * ks) * (dp - dm);
-    a = s - r;
-    b = real(1) + real(2) * r;
-    c = -s - r;
-}
-
 // Shared-memory slot of line element k: element j of segment t sits at
 // j * sp + t (sp odd), so the threads of a warp sweeping their segments touch
 // consecutive words at every step (no bank conflicts).
@@ -1124,7 +1114,7 @@ __device__ __forceinline__ void t_row(const LineArgs<real> &A, int k, real dm, r
         b = real(1);
         return;
     }
-    coef23_folded(A.kr, A.ks, dd, dm, dp, a, b, c);
+    coef23(A.c.B3, A.hrh, A.srh, A.rh2, dd, dm, dp, a, b, c);
     if (k == 0) {
         if (!lo_sine) b -= a;
         else if (rk) *rk -= a * lo_inc;
@@ -1240,7 +1230,7 @@ __device__ __forceinline__ void line_solve_reg(const LineArgs<real> &A, int line
             real ta[M + 2], tb[M + 2], tc[M + 2];   // T's rows f - 1 .. f + M
 #pragma unroll
             for (int j = 0; j < M + 2; j++)
-                coef23_folded(A.kr, A.ks, dv[j + 1], dv[j], dv[j + 2], ta[j], tb[j], tc[j]);
+                coef23(A.c.B3, A.hrh, A.srh, A.rh2, dv[j + 1], dv[j], dv[j + 2], ta[j], tb[j], tc[j]);
             if (f == 0 || at_end) {
 #pragma unroll
                 for (int j = 0; j < M + 2; j++)
@@ -1257,7 +1247,7 @@ __device__ __forceinline__ void line_solve_reg(const LineArgs<real> &A, int line
         } else {
 #pragma unroll
             for (int j = 0; j < M; j++)
-                coef23_folded(A.kr, A.ks, dv[j + 2], dv[j + 1], dv[j + 3], ra[j], rb[j], rc[j]);
+                coef23(A.c.B3, A.hrh, A.srh, A.rh2, dv[j + 2], dv[j + 1], dv[j + 3], ra[j], rb[j], rc[j]);
             // the makers' ghost increments (t^{n+1} - t^n) at the line's ends
             // and the coefficients that carry them to the right side
             real lo_inc = real(0), hi_inc = real(0), a_lo = real(0), c_hi = real(0);
@@ -1289,21 +1279,23 @@ __device__ __forceinline__ void line_solve_reg(const LineArgs<real> &A, int line
         }
         // Thomas on rows f .. f + M - 2 against (r, -a_f e_0, -c e_last): the
         // rows' own factors and the couplings' columns first, which need no
-        // right side, so that its load is in flight meanwhile; ra becomes
-        // a / pivot, rb 1 / pivot and rc c / pivot
+        // right side, so that its load is in flight meanwhile; rb becomes
+        // 1 / pivot and rc c / pivot.  The order of the operations is part of
+        // the result: the matrix is ill-conditioned for smooth solutions by
+        // about 4 (B + 1/3) d^2 / dx^2 (several hundred on fine grids), and by
+        // as much the roundings of the elimination and of Eq. 23's
+        // coefficients grow in the discharges' increments.
         real y[m1], uu[m1], vv[m1];
         real Y = real(0), U = real(0), V = real(0);
         const real al = ra[m1], bl = rb[m1], cl = rc[m1];
         rb[0] = rcp_r(rb[0]);
-        ra[0] *= rb[0];
         rc[0] *= rb[0];
-        uu[0] = -ra[0];
+        uu[0] = -ra[0] * rb[0];
 #pragma unroll
         for (int j = 1; j < m1; j++) {
             rb[j] = rcp_r(rb[j] - ra[j] * rc[j - 1]);
-            ra[j] *= rb[j];
             rc[j] *= rb[j];
-            uu[j] = -ra[j] * uu[j - 1];
+            uu[j] = -ra[j] * uu[j - 1] * rb[j];
         }
         vv[m1 - 1] = -rc[m1 - 1];
 #pragma unroll
@@ -1313,7 +1305,7 @@ __device__ __forceinline__ void line_solve_reg(const LineArgs<real> &A, int line
         }
         y[0] = r[0] * rb[0];
 #pragma unroll
-        for (int j = 1; j < m1; j++) y[j] = r[j] * rb[j] - ra[j] * y[j - 1];
+        for (int j = 1; j < m1; j++) y[j] = (r[j] - ra[j] * y[j - 1]) * rb[j];
 #pragma unroll
         for (int j = m1 - 2; j >= 0; j--) y[j] -= rc[j] * y[j + 1];
         // the separator's row in (s_{t-1}, s_t, s_{t+1}): the next thread's

@@ -1,9 +1,10 @@
 """The step kernels at the sizes and depths where their variants can go wrong,
 against the FP64 oracle: films around the depth from which Eq. 14's velocity
-factor is 1/h, tile edges and remainders, and non-finite states.
+factor is 1/h, tile edges and remainders, and non-finite states; the line
+solves' FP64 digits.
 
-Bars: those of the parity tests, relative L2 1e-10 (FP64) and 1e-4 (FP32) for
-eta, ten times that for P and Q.
+Bars of the comparisons with the oracle: those of the parity tests, relative L2
+1e-10 (FP64) and 1e-4 (FP32) for eta, ten times that for P and Q.
 """
 import numpy as np
 import pytest
@@ -91,3 +92,36 @@ def test_carries_correctors_and_shallow_water_across_tiles(K, model):
         s.sides[side] = sc.Side(sc.SINE, 0, ((0.02, 3.0, 0.3 + side, 0.1 * side),))
     for prec in ("f32", "f64"):
         _match(s, prec, 6)
+
+
+@pytest.mark.parametrize("nx,ny,dx,d", [(256, 32, 0.05, 1.0), (512, 64, 0.1, 1.0), (200, 40, 0.03, 0.32)])
+def test_line_solves_keep_fp64_digits(nx, ny, dx, d):
+    """One Euler step of a hump at rest: P is the x-solves' increment itself,
+    against the same systems solved in extended precision.  A system of
+    r = (B + 1/3) d^2 / dx^2 is ill-conditioned by 1 + 4 r for smooth solutions;
+    the elimination in the kernel's order leaves 0.05 eps (1 + 4 r) or less, one
+    on rows scaled by their pivots with coefficients folded per line twice as
+    much (0.10, 0.10 and 0.05): the bar lies between."""
+    from paper_1611_05984_gb300 import celeris
+    wide = np.longdouble
+    s = sc.flat_basin(nx, ny, dx, d, 0.2 * dx / np.sqrt(9.81 * d))
+    s.w0 = np.broadcast_to(0.1 * np.exp(-(((np.arange(nx) + 0.5) / nx - 0.4) * 12.0) ** 2), (ny, nx)).copy()
+    g = celeris.from_scenario(s, dtype=torch.float64)
+    g.step(1)
+    rhs = g.field("U").cpu().numpy().astype(wide)
+    P = g.state()[1].cpu().numpy()
+    r = (wide(s.Bd) + wide(1) / wide(3)) * wide(d) * wide(d) / (wide(dx) * wide(dx))
+    b = np.full(nx, 1 + 2 * r)
+    b[0] += r
+    b[-1] += r
+    c, x = np.zeros(nx, wide), np.zeros_like(rhs)
+    for k in range(nx):
+        a = -r if k else wide(0)
+        pivot = b[k] - a * c[k - 1]
+        c[k] = -r / pivot
+        x[:, k] = (rhs[:, k] - a * x[:, k - 1]) / pivot
+    for k in range(nx - 2, -1, -1):
+        x[:, k] -= c[k] * x[:, k + 1]
+    err = float(np.linalg.norm((P - x).astype(np.float64)) / np.linalg.norm(x.astype(np.float64)))
+    bar = (0.035 if d < 1.0 else 0.075) * 2.0 ** -53 * float(1 + 4 * r)
+    assert err <= bar, f"{err:.2e} above {bar:.2e}"
