@@ -167,11 +167,14 @@ __device__ __forceinline__ real bbar_at(const real *Bc, const Geo &g, int i, int
                      corner(Bc, g, i + 1, j + 1));
 }
 
+constexpr float kRoot2 = 1.4142135623730951f;
+
 // The FP32 stencil's constants twice over, as its two-cell operations take
 // them (a constant then costs one 64-bit load instead of two moves).
 enum {
-    kcTh2, kcQ, kcMQ, kcHalf, kcTwo, kcMTwo, kcMThree, kcG, kcWs, kcRdx, kcRdy, kcMHgx, kcMHgy, kcMFric, kcRdx2, kcRdy2,
-    kcKx, kcKy, kcC6, kcB3xy, kcDt, kcAb0, kcAb1, kcAb2, kcAm0, kcAm1, kcAm2, kcAm3, kcCount
+    kcTh2, kcQ, kcMQ, kcHalf, kcOne, kcTwo, kcMOne, kcMTwo, kcMThree, kcRoot2, kcHalfG, kcMHalfG, kcWs, kcRdx, kcRdy, kcFric,
+    kcHrdx, kcHrdy, kcRdx2, kcRdy2, kcRdxdy4, kcRdx3h, kcRdy3h, kcRdxdy2h, kcRdx2dyh, kcBg, kcSixth, kcB3, kcDt, kcC12,
+    kcC24, kc9C24, kc23C12, kcM16C12, kc5C12, kc23, kcM16, kc5, kc19, kcM5, kcCount
 };
 template <typename real>
 struct PairConst {};
@@ -182,9 +185,11 @@ struct PairConst<float> {
 inline void make_pairs(const Coef<double> &, PairConst<double> &) {}
 inline void make_pairs(const Coef<float> &c, PairConst<float> &p)
 {
-    const float v[kcCount] = {c.th2, 0.25f, -0.25f, 0.5f, 2.f, -2.f, -3.f, c.g, c.ws, c.rdx, c.rdy, -c.hgx, -c.hgy, -c.fric,
-                              c.rdx2, c.rdy2, c.Kx, c.Ky, c.c6, c.B3xy, c.dt, c.ab[0], c.ab[1], c.ab[2], c.am[0],
-                              c.am[1], c.am[2], c.am[3]};
+    const float c12 = c.dt * (1.f / 12.f), c24 = c.dt * (1.f / 24.f);
+    const float v[kcCount] = {
+        c.th2, 0.25f, -0.25f, 0.5f, 1.f, 2.f, -1.f, -2.f, -3.f, kRoot2, 0.5f * c.g, -0.5f * c.g, c.ws, c.rdx, c.rdy, c.fric,
+        c.hrdx, c.hrdy, c.rdx2, c.rdy2, c.rdxdy4, c.rdx3h, c.rdy3h, c.rdxdy2h, c.rdx2dyh, c.Bd * c.g, c.sixth, c.B3, c.dt,
+        c12, c24, 9.f * c24, 23.f * c12, -16.f * c12, 5.f * c12, 23.f, -16.f, 5.f, 19.f, -5.f};
     for (int k = 0; k < kcCount; k++) p.v[k] = make_float2(v[k], v[k]);
 }
 

@@ -148,11 +148,6 @@ __device__ __forceinline__ double sqrt_r(double x)
 __device__ __forceinline__ float rsqrt_r(float x) { return rsqrtf(x); }
 
 // sqrt(x) and c / x' for x = g h, c = g: the celerity and 1/h from one root.
-__device__ __forceinline__ void root_and_inverse(float g, float h, float gh, float &s, float &ih)
-{
-    s = sqrtf(gh);
-    ih = rcp_r(h);
-}
 __device__ __forceinline__ void root_and_inverse(double g, double h, double gh, double &s, double &ih)
 {
     const double r = rsqrt_r(gh);
@@ -196,12 +191,6 @@ __device__ __forceinline__ float max_zero(float a, float b)
 {
     float d;
     asm("max.ftz.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(0.f));
-    return d;
-}
-__device__ __forceinline__ float min_zero(float a, float b)
-{
-    float d;
-    asm("min.ftz.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(0.f));
     return d;
 }
 __device__ __forceinline__ double max_zero(double a, double b)

@@ -7,18 +7,16 @@
 //     multiply-adds on both at once (.f32x2), 64-bit loads and stores of
 //     shared and global memory, and one set of addresses, branches and loop
 //     counts for two cells;
-//   * a warp marches up its rows, so the reconstruction and fluxes along y,
-//     the differences of the rows below and the bed's corner sums stay in
-//     registers; a cell's x-fluxes come from its own reconstruction and its
-//     left neighbour's (shuffles), and none goes through shared memory;
-//   * the mixed and third differences of Eq. 10-13 are differences between
-//     rows of each row's own x-differences.
+//   * a warp marches up its rows, so the reconstruction and fluxes along y and
+//     the depth of the row below stay in registers; a cell's x-fluxes come
+//     from its own reconstruction and its left neighbour's (shuffles), and
+//     none goes through shared memory.
 // The faces at the tile's west and east edges, which need cells of the
 // neighbouring tiles' lanes, are computed first, one (side, row) per lane.
 //
 // A face's flux does not depend on which warp or variant computes it (the
-// row's one branch only skips what it would not do), so tiles of different
-// heights give the same bits.
+// row's one branch, on a negative depth, skips a fix that would change
+// nothing), so tiles of different heights give the same bits.
 //
 // Per cell about 455 thread instructions in the predictor and 410 in the
 // corrector (865 and 800 with a cell per thread and the fluxes in shared
@@ -34,6 +32,7 @@ namespace cel {
 namespace {
 
 using pk = unsigned long long;   // two floats: the cells x and x + 1
+constexpr float kLeastNormal = 1.17549435e-38f;   // a speed's reciprocal stays finite (smaller ones are flushed to 0)
 
 __device__ __forceinline__ pk mk(float a, float b)
 {
@@ -54,7 +53,6 @@ __device__ __forceinline__ float py_(pk v)
     un(v, a, b);
     return b;
 }
-__device__ __forceinline__ pk kc(const StencilArgs<float> &A, int k) { return *reinterpret_cast<const pk *>(&A.kk.v[k]); }
 __device__ __forceinline__ pk add2(pk a, pk b)
 {
     pk r;
@@ -79,12 +77,49 @@ __device__ __forceinline__ pk fma2(pk a, pk b, pk c)
     asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
 }
-__device__ __forceinline__ float min4(float a, float b, float c, float d)
+// f of each half
+template <typename F>
+__device__ __forceinline__ pk each(pk v, const F &f)
 {
-    float r;
-    asm("min.ftz.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return fminf(r, d);
+    float a, b;
+    un(v, a, b);
+    return mk(f(a), f(b));
 }
+__device__ __forceinline__ pk max2(pk v, float m) { return each(v, [=](float x) { return fmaxf(x, m); }); }
+__device__ __forceinline__ pk max_zero2(pk v, pk w)
+{
+    float a, b, c, d;
+    un(v, a, b);
+    un(w, c, d);
+    return mk(max_zero(a, c), max_zero(b, d));
+}
+__device__ __forceinline__ pk sqrt2(pk v) { return each(v, [](float x) { return sqrtf(x); }); }
+__device__ __forceinline__ pk rsqrt2(pk v) { return each(v, [](float x) { return rsqrtf(x); }); }
+__device__ __forceinline__ pk rcp2(pk v) { return each(v, [](float x) { return rcp_r(x); }); }
+__device__ __forceinline__ pk cbrt2(pk v) { return each(v, [](float x) { return cbrt_r(x); }); }
+
+// The same operations on one cell, so that the arithmetic below is stated once
+// for pairs and for single cells and gives both the same bits.
+__device__ __forceinline__ float add2(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub2(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float mul2(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float fma2(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float max2(float v, float m) { return fmaxf(v, m); }
+__device__ __forceinline__ float max_zero2(float v, float w) { return max_zero(v, w); }
+__device__ __forceinline__ float sqrt2(float v) { return sqrtf(v); }
+__device__ __forceinline__ float rsqrt2(float v) { return rsqrtf(v); }
+__device__ __forceinline__ float rcp2(float v) { return rcp_r(v); }
+__device__ __forceinline__ float cbrt2(float v) { return cbrt_r(v); }
+
+// Constant k of the arguments
+template <typename V>
+__device__ __forceinline__ V kc(const StencilArgs<float> &A, int k)
+{
+    if constexpr (sizeof(V) == 8) return *reinterpret_cast<const pk *>(&A.kk.v[k]);
+    else return A.kk.v[k].x;
+}
+__device__ __forceinline__ pk kc(const StencilArgs<float> &A, int k) { return kc<pk>(A, k); }
+
 __device__ __forceinline__ pk ldp(const float *p) { return *reinterpret_cast<const pk *>(p); }
 // The same, read again even where the value was read before.
 __device__ __forceinline__ pk ldv(const float *p)
@@ -93,9 +128,11 @@ __device__ __forceinline__ pk ldv(const float *p)
     asm volatile("ld.volatile.shared.b64 %0, [%1];" : "=l"(r) : "r"((unsigned)__cvta_generic_to_shared(p)));
     return r;
 }
-// pair k of a global array
-__device__ __forceinline__ pk ldo(const float *p, unsigned k) { return reinterpret_cast<const pk *>(p)[k]; }
-__device__ __forceinline__ void sto(float *p, unsigned k, pk v) { reinterpret_cast<pk *>(p)[k] = v; }
+// pair or value k of a global array
+template <typename V>
+__device__ __forceinline__ V ldo(const float *p, unsigned k) { return reinterpret_cast<const V *>(p)[k]; }
+template <typename V>
+__device__ __forceinline__ void sto(float *p, unsigned k, V v) { reinterpret_cast<V *>(p)[k] = v; }
 
 constexpr int kPW = kPairCols, kPWarps = kPairWarps;
 constexpr int kPThreads = 32 * kPWarps;
@@ -116,83 +153,98 @@ struct PairSmem {
     uint32_t col[kPW];           // dry bits per column
 };
 
-// The history a stage reads for two cells (Carry, twice).
-struct CarryPair {
-    pk a, b, r1, r2, p1, p2, Y;
+// The history a stage reads (Carry), of two cells or one.
+template <typename V>
+struct CarryV {
+    V a, b, r1, r2, p1, p2, Y;
 };
 
-template <int kSpec>
-__device__ __forceinline__ CarryPair load_carry_pair(const StencilArgs<float> &A, int v, unsigned k)
+template <typename V, int kSpec>
+__device__ __forceinline__ CarryV<V> load_carry_v(const StencilArgs<float> &A, int v, unsigned k)
 {
     const int kind = kSpec == 1 ? kAB3 : (kSpec == 2 ? kAM4 : A.kind);
     const bool ring = kSpec != 0 ? true : A.ring != 0;
-    CarryPair c;
+    CarryV<V> c;
     c.a = c.b = c.r1 = c.r2 = c.p1 = c.p2 = c.Y = 0;
     if (kind == kAM4) {
-        c.Y = ldo(A.Y[v], k);
+        c.Y = ldo<V>(A.Y[v], k);
     } else if (ring) {
         if (kind == kAB3) {
-            c.r1 = ldo(A.R1[v], k);
-            c.r2 = ldo(A.R2[v], k);
+            c.r1 = ldo<V>(A.R1[v], k);
+            c.r2 = ldo<V>(A.R2[v], k);
         }
         if (v > 0 && kind != kEuler0) {
-            c.p1 = ldo(A.F1[v], k);
-            if (kind == kAB3) c.p2 = ldo(A.F2[v], k);
+            c.p1 = ldo<V>(A.F1[v], k);
+            if (kind == kAB3) c.p2 = ldo<V>(A.F2[v], k);
         }
     } else if (kind == kEuler1) {
-        c.a = ldo(A.a[v], k);
+        c.a = ldo<V>(A.a[v], k);
     } else if (kind == kAB3) {
-        c.a = ldo(A.a[v], k);
-        c.b = ldo(A.b[v], k);
+        c.a = ldo<V>(A.a[v], k);
+        c.b = ldo<V>(A.b[v], k);
     }
     return c;
 }
 
-// advance() for two cells; the history is written where ok.
-template <int kSpec>
-__device__ __forceinline__ pk advance_pair(const StencilArgs<float> &A, int v, pk X0, pk R, pk Phi, unsigned k,
-                                           const CarryPair &c, bool ok)
+// The single-precision arithmetic, on two cells or one (V).
+//
+// The order of every operation is part of the result, and a product that is
+// rounded on its own before a sum is the addend of a fused multiply-add (the
+// compiler may contract a plain sum of two cells with it).  Where a discharge is a small difference of
+// large terms (the cross-tank one around an island, of the pressure 1/2 g h^2,
+// the bed slope and the third differences of eta) its digits are this order's
+// rounding errors over dx: on a 1178 x 1178 island another order, as close to
+// 64 bits, parted from this one by 3.7e-5 of the discharge's norm and 2.4e-3
+// of its root mean square.  tests/test_gpu_step_kernels.py pins the bits.
+
+// advance(): the increment of U* or V*; of w the increment in the Euler stages
+// and w itself in the others (kSpec 1 and 2).  The history is written where ok.
+template <typename V, int kSpec>
+__device__ __forceinline__ V advance_v(const StencilArgs<float> &A, int v, V X0, V R, V Phi, unsigned k,
+                                       const CarryV<V> &c, bool ok)
 {
     const int kind = kSpec == 1 ? kAB3 : (kSpec == 2 ? kAM4 : A.kind);
     const bool ring = kSpec != 0 ? true : A.ring != 0;
     if (kind == kAM4) {
-        const pk s = fma2(kc(A, kcAm0), R, c.Y);
+        const V s = fma2(kc<V>(A, kc9C24), R, c.Y);
         return v > 0 ? add2(s, Phi) : s;
     }
-    pk D;
+    V D;
     if (ring) {
         if (ok) {
             sto(A.R0[v], k, R);
             if (v > 0) sto(A.F0[v], k, Phi);
         }
         if (kind != kAB3) {
-            D = mul2(kc(A, kcDt), R);
-            if (kind == kEuler1 && v > 0) D = add2(D, sub2(Phi, c.p1));
+            if (kind == kEuler1 && v > 0) D = fma2(kc<V>(A, kcDt), R, sub2(Phi, c.p1));
+            else D = mul2(kc<V>(A, kcDt), R);
         } else {
-            D = fma2(kc(A, kcAb2), c.r2, fma2(kc(A, kcAb1), c.r1, mul2(kc(A, kcAb0), R)));
-            pk y = fma2(kc(A, kcAm3), c.r2, fma2(kc(A, kcAm2), c.r1, mul2(kc(A, kcAm1), R)));
+            const V s = fma2(kc<V>(A, kc5), c.r2, fma2(kc<V>(A, kc23), R, mul2(kc<V>(A, kcM16), c.r1)));
+            const V t = add2(fma2(kc<V>(A, kc19), R, mul2(kc<V>(A, kcM5), c.r1)), c.r2);
+            V y;
             if (v > 0) {
-                D = add2(D, fma2(kc(A, kcTwo), Phi, fma2(kc(A, kcMThree), c.p1, c.p2)));
-                y = sub2(y, Phi);
+                D = add2(fma2(kc<V>(A, kcMThree), c.p1, fma2(kc<V>(A, kcTwo), Phi, mul2(kc<V>(A, kcC12), s))), c.p2);
+                y = fma2(kc<V>(A, kcMOne), Phi, mul2(kc<V>(A, kcC24), t));
             } else {
-                y = add2(X0, y);
+                D = fma2(kc<V>(A, kcOne), X0, mul2(kc<V>(A, kcC12), s));   // w itself
+                y = fma2(kc<V>(A, kcC24), t, X0);
             }
             if (ok) sto(A.Y[v], k, y);
         }
         return D;
     }
-    pk na;
+    V na;
     if (kind == kEuler0) {
-        D = mul2(kc(A, kcDt), R);
+        D = mul2(kc<V>(A, kcDt), R);
         na = Phi;
     } else {
-        if (kind == kEuler1) D = add2(mul2(kc(A, kcDt), R), sub2(Phi, c.a));
-        else D = add2(fma2(kc(A, kcTwo), Phi, mul2(kc(A, kcAb0), R)), add2(c.a, c.b));
-        na = fma2(kc(A, kcMThree), Phi, mul2(kc(A, kcAb1), R));
+        if (kind == kEuler1) D = fma2(kc<V>(A, kcDt), R, sub2(Phi, c.a));
+        else D = add2(fma2(kc<V>(A, kcTwo), Phi, mul2(kc<V>(A, kc23C12), R)), add2(c.a, c.b));
+        na = fma2(kc<V>(A, kcM16C12), R, mul2(kc<V>(A, kcMThree), Phi));
     }
     if (ok) {
         sto(A.a[v], k, na);
-        sto(A.b[v], k, fma2(kc(A, kcAb2), R, Phi));
+        sto(A.b[v], k, fma2(kc<V>(A, kc5C12), R, Phi));
     }
     return D;
 }
@@ -251,96 +303,82 @@ __device__ __forceinline__ void fix_pair(pk w, pk Blo, pk Bhi, pk &lo, pk &hi, p
     dhi = mk(h0, h1);
 }
 
-// KP07 step 3 on two faces (face_flux_step): left states L, depths hL, right
-// states R, depths hR; H = (mass, normal, tangential momentum).  kWet: every
-// depth reaches eps^(1/4) (no branch); else each face takes its own form.
-template <bool kWet>
-__device__ __forceinline__ void flux_pair(const StencilArgs<float> &A, const pk L[3], pk hL, const pk R[3], pk hR,
-                                          pk H[3])
+// Eq. 14's factor of a depth >= 0 (desing).
+template <typename V>
+__device__ __forceinline__ V desing_v(const StencilArgs<float> &A, V h)
 {
-    float l0, l1, r0, r1, gl0, gl1, gr0, gr1;
-    un(hL, l0, l1);
-    un(hR, r0, r1);
-    const pk ghL = mul2(kc(A, kcG), hL), ghR = mul2(kc(A, kcG), hR);
-    un(ghL, gl0, gl1);
-    un(ghR, gr0, gr1);
-    const pk sL = mk(sqrtf(gl0), sqrtf(gl1)), sR = mk(sqrtf(gr0), sqrtf(gr1));
-    pk nL = L[1], tL = L[2], nR = R[1], tR = R[2], uL, vL, uR, vR;
-    if (kWet) {
-        const pk kL = mk(rcp_r(l0), rcp_r(l1)), kR = mk(rcp_r(r0), rcp_r(r1));
-        uL = mul2(kL, nL);
-        vL = mul2(kL, tL);
-        uR = mul2(kR, nR);
-        vR = mul2(kR, tR);
-    } else {
-        // a face with both depths at eps^(1/4) or above as in the other form
-        const bool w0 = fminf(l0, r0) >= A.c.hwet, w1 = fminf(l1, r1) >= A.c.hwet;
-        const float eps = A.c.eps;
-        const pk kL = mk(w0 ? rcp_r(l0) : desing(l0, eps), w1 ? rcp_r(l1) : desing(l1, eps));
-        const pk kR = mk(w0 ? rcp_r(r0) : desing(r0, eps), w1 ? rcp_r(r1) : desing(r1, eps));
-        uL = mul2(kL, nL);
-        vL = mul2(kL, tL);
-        uR = mul2(kR, nR);
-        vR = mul2(kR, tR);
-        auto pick = [&](pk &q, pk k) {
-            float a, b, c, d;
-            un(q, a, b);
-            un(k, c, d);
-            q = mk(w0 ? a : c, w1 ? b : d);
-        };
-        pick(nL, mul2(hL, uL));
-        pick(tL, mul2(hL, vL));
-        pick(nR, mul2(hR, uR));
-        pick(tR, mul2(hR, vR));
-    }
-    float p0, p1, q0, q1;
-    un(add2(uL, sL), p0, p1);
-    un(add2(uR, sR), q0, q1);
-    const pk ap = mk(max_zero(p0, q0), max_zero(p1, q1));
-    un(sub2(uL, sL), p0, p1);
-    un(sub2(uR, sR), q0, q1);
-    const pk am = mk(min_zero(p0, q0), min_zero(p1, q1));
-    float d0, d1;
-    un(sub2(am, ap), d0, d1);   // -(a+ - a-)
-    // where both sides are dry (Reading A-F1) all terms are 0 and so is the flux
-    const pk ninv = kWet ? mk(rcp_r(d0), rcp_r(d1)) : mk(rcp_r(fminf(d0, -1e-30f)), rcp_r(fminf(d1, -1e-30f)));
-    const pk beta = mul2(am, ninv), ab = mul2(ap, beta);
-    const pk FL1 = fma2(kc(A, kcHalf), mul2(ghL, hL), mul2(nL, uL)), FR1 = fma2(kc(A, kcHalf), mul2(ghR, hR), mul2(nR, uR));
-    const pk FL2 = mul2(nL, vL), FR2 = mul2(nR, vR);
-    H[0] = fma2(ab, sub2(L[0], R[0]), fma2(beta, sub2(nR, nL), nL));
-    H[1] = fma2(ab, sub2(nL, nR), fma2(beta, sub2(FR1, FL1), FL1));
-    H[2] = fma2(ab, sub2(tL, tR), fma2(beta, sub2(FR2, FL2), FL2));
+    const V h2 = mul2(h, h), h4 = mul2(h2, h2);
+    return mul2(mul2(kc<V>(A, kcRoot2), h), rsqrt2(fma2(kc<V>(A, kcOne), h4, max2(h4, A.c.eps))));
 }
 
-// Friction's factor of (P, Q), negated: two cells with depths hb.
-template <bool kWet>
-__device__ __forceinline__ pk friction_pair(const StencilArgs<float> &A, int law, pk hb, pk P, pk Q)
+// KP07 step 3: left states L = (w, normal, tangential discharge) and depths
+// hL >= 0, right states R, depths hR; H = (mass, normal, tangential momentum).
+template <typename V>
+__device__ __forceinline__ void flux_v(const StencilArgs<float> &A, const V L[3], V hL, const V R[3], V hR, V H[3])
 {
-    float h0, h1, m0, m1;
-    un(hb, h0, h1);
-    un(fma2(Q, Q, mul2(P, P)), m0, m1);
-    pk k;
-    if (kWet) {
-        k = mk(rcp_r(h0), rcp_r(h1));
-    } else {
-        const float eps = A.c.eps, hw = A.c.hwet;
-        k = mk(h0 >= hw ? rcp_r(h0) : desing(fmaxf(h0, 0.f), eps), h1 >= hw ? rcp_r(h1) : desing(fmaxf(h1, 0.f), eps));
-    }
-    pk f = mul2(mul2(k, k), mk(sqrtf(m0), sqrtf(m1)));
-    if (law == kFricManning) {
-        float k0, k1;
-        un(k, k0, k1);
-        f = mul2(f, mk(cbrt_r(k0), cbrt_r(k1)));
-    }
-    return mul2(f, kc(A, kcMFric));
+    const V kL = desing_v(A, hL), kR = desing_v(A, hR);
+    const V uL = mul2(kL, L[1]), vL = mul2(kL, L[2]), uR = mul2(kR, R[1]), vR = mul2(kR, R[2]);
+    const V nL = mul2(hL, uL), nR = mul2(hR, uR);
+    const V gL = mul2(kc<V>(A, kcHalfG), hL), gR = mul2(kc<V>(A, kcHalfG), hR);
+    const V sL = sqrt2(add2(gL, gL)), sR = sqrt2(add2(gR, gR));
+    const V ap = max_zero2(add2(uL, sL), add2(uR, sR)), nam = max_zero2(sub2(sL, uL), sub2(sR, uR));   // a+, -a-
+    // where both sides are dry (Reading A-F1) every term is 0 and so is the flux
+    const V inv = rcp2(max2(add2(ap, nam), kLeastNormal)), nab = mul2(ap, nam);
+    const V FL1 = fma2(gL, hL, mul2(nL, uL)), FR1 = fma2(gR, hR, mul2(nR, uR));
+    H[0] = mul2(inv, fma2(nab, sub2(L[0], R[0]), fma2(ap, nL, mul2(nam, nR))));
+    H[1] = mul2(inv, fma2(nab, sub2(nL, nR), fma2(ap, FL1, mul2(nam, FR1))));
+    H[2] = mul2(inv, fma2(nab, fma2(mul2(kc<V>(A, kcMOne), hR), vR, mul2(hL, vL)),
+                          fma2(ap, mul2(nL, vL), mul2(nam, mul2(nR, vR)))));
 }
 
-__device__ __forceinline__ float least(pk a, pk b)
+// Friction (Eq. 31-32) subtracted from F and G of a cell of depth hb.
+template <typename V>
+__device__ __forceinline__ void friction_v(const StencilArgs<float> &A, int law, V hb, V P, V Q, V &F, V &G)
 {
-    float a0, a1, b0, b1;
-    un(a, a0, a1);
-    un(b, b0, b1);
-    return min4(a0, a1, b0, b1);
+    const V k = desing_v(A, max2(hb, 0.f)), nk = mul2(kc<V>(A, kcMOne), k);
+    V fc = kc<V>(A, kcFric);
+    if (law == kFricManning) fc = mul2(fc, cbrt2(k));
+    const V mag = sqrt2(fma2(P, P, mul2(Q, Q)));
+    F = fma2(mul2(mul2(mul2(fc, P), mag), k), nk, F);
+    G = fma2(mul2(mul2(mul2(fc, Q), mag), k), nk, G);
+}
+
+// A cell's value c with its neighbours' (for eta two cells out along the axes).
+template <typename V>
+struct Around {
+    V c, e, w, n, s, ne, nw, se, sw, ee, ww, nn, ss;
+};
+
+// Eq. 10-11's dispersive terms added to F and G: w around the cell, its depth
+// d and the depth's gradient.
+template <typename V>
+__device__ __forceinline__ void eta_terms_v(const StencilArgs<float> &A, const Around<V> &q, V d, V ddx, V ddy, V &F, V &G)
+{
+    const V two = kc<V>(A, kcTwo), mtwo = kc<V>(A, kcMTwo);
+    const V K2 = mul2(mul2(kc<V>(A, kcBg), d), d), K3 = mul2(K2, d);
+    const V exx = mul2(add2(fma2(mtwo, q.c, q.e), q.w), kc<V>(A, kcRdx2));
+    const V eyy = mul2(add2(fma2(mtwo, q.c, q.n), q.s), kc<V>(A, kcRdy2));
+    const V exy = mul2(add2(sub2(sub2(q.ne, q.se), q.nw), q.sw), kc<V>(A, kcRdxdy4));
+    const V exxx = sub2(fma2(two, q.w, fma2(mtwo, q.e, q.ee)), q.ww);   // the third differences undivided
+    const V eyyy = sub2(fma2(two, q.s, fma2(mtwo, q.n, q.nn)), q.ss);
+    const V exyy = sub2(add2(fma2(mtwo, q.e, q.ne), q.se), add2(fma2(mtwo, q.w, q.nw), q.sw));
+    const V exxy = sub2(add2(fma2(mtwo, q.n, q.ne), q.nw), add2(fma2(mtwo, q.s, q.se), q.sw));
+    const V x3 = fma2(exxx, kc<V>(A, kcRdx3h), mul2(exyy, kc<V>(A, kcRdxdy2h)));
+    const V y3 = fma2(eyyy, kc<V>(A, kcRdy3h), mul2(exxy, kc<V>(A, kcRdx2dyh)));
+    const V x2 = fma2(ddx, fma2(two, exx, eyy), mul2(ddy, exy)), y2 = fma2(ddy, fma2(two, eyy, exx), mul2(ddx, exy));
+    F = add2(F, fma2(K3, x3, mul2(K2, x2)));
+    G = add2(G, fma2(K3, y3, mul2(K2, y2)));
+}
+
+// Eq. 12-13's mixed terms: F* from Q, G* from P around the cell (no second
+// neighbours).
+template <typename V>
+__device__ __forceinline__ V mixed_term_v(const StencilArgs<float> &A, const Around<V> &q, V d, V ddx, V ddy)
+{
+    const V qx = mul2(sub2(q.e, q.w), kc<V>(A, kcHrdx)), qy = mul2(sub2(q.n, q.s), kc<V>(A, kcHrdy));
+    const V qxy = mul2(add2(sub2(sub2(q.ne, q.se), q.nw), q.sw), kc<V>(A, kcRdxdy4)), sixth = kc<V>(A, kcSixth);
+    return fma2(mul2(mul2(kc<V>(A, kcB3), d), d), qxy,
+                fma2(mul2(mul2(d, ddy), qx), sixth, mul2(mul2(mul2(d, ddx), qy), sixth)));
 }
 
 // A lane's pair of values at its cells' west faces, from its left neighbour's
@@ -416,25 +454,26 @@ __device__ __forceinline__ SideRow side_row(const float *w, const float *P, cons
     return s;
 }
 
-// The x-differences of a row that the rows beside it combine (central
-// differences of w, P and Q, second difference of w, undivided).
-struct DiffRow {
-    pk w, ww, P, Q;
-};
-
-__device__ __forceinline__ DiffRow diff_row(const SideRow &s, pk w, pk P, pk Q)
+// The pairs around the pair v at p in shared memory (rows kStrideOf apart, n
+// and s those above and below), read again (ldv).
+template <int kStrideOf>
+__device__ __forceinline__ Around<pk> aroundv(const float *p, pk v, pk n, pk s)
 {
-    DiffRow d;
-    float a, b;
-    un(w, a, b);
-    const pk m = mk(s.wl, a), p = mk(b, s.wr);
-    d.w = sub2(p, m);
-    d.ww = sub2(sub2(p, w), sub2(w, m));
-    un(P, a, b);
-    d.P = sub2(mk(b, s.pr), mk(s.pl, a));
-    un(Q, a, b);
-    d.Q = sub2(mk(b, s.qr), mk(s.ql, a));
-    return d;
+    Around<pk> q;
+    auto sides = [](const float *r, pk c, pk &e, pk &w, pk &ee, pk &ww) {
+        ww = ldv(r - 2);
+        ee = ldv(r + 2);
+        e = mk(py_(c), px_(ee));
+        w = mk(py_(ww), px_(c));
+    };
+    pk beyond[2];
+    q.c = v;
+    q.n = n;
+    q.s = s;
+    sides(p, v, q.e, q.w, q.ee, q.ww);
+    sides(p + kStrideOf, n, q.ne, q.nw, beyond[0], beyond[1]);
+    sides(p - kStrideOf, s, q.se, q.sw, beyond[0], beyond[1]);
+    return q;
 }
 
 __device__ __forceinline__ uint32_t spread_bits(uint32_t x)   // bit k of the low half to bit 2k
@@ -647,7 +686,7 @@ __device__ __forceinline__ void stencil_tile_pair(const StencilArgs<float> &A, c
         fs.open(C.th2, q0, q1);
         fs.next(C.th2, q2, 0.5f * (c0 + e0), Bf, lo, hi, dl, dh);
         fs.next(C.th2, q3, Bf, 0.5f * (c2 + e2), lo2, hi2, dl2, dh2);
-        face_flux_step(C.g, C.eps, C.hwet, hi[0], hi[1], hi[2], dh, lo2[0], lo2[1], lo2[2], dl2, H);
+        flux_v<float>(A, hi, dh, lo2, dl2, H);
         // the cell beyond: f - 1 on the west, f on the east
         const float Bb = side ? cell_bbar(c1, c2, e1, e2) : cell_bbar(c0, c1, e0, e1);
         sm.edge[side][r] = make_float4(H[0], H[1], H[2], fmaxf(C.ws - Bb, 0.f));
@@ -656,7 +695,7 @@ __device__ __forceinline__ void stencil_tile_pair(const StencilArgs<float> &A, c
 
     // ---- 4. the rows.  What a row shares with the next and is dearer to
     //         read again than to keep: the next row's cells, the fluxes and
-    //         high sides along y, the x-differences of the row below.
+    //         high sides along y, the depth of the row below.
     const float ws = C.ws;
     const bool bsnq = A.phy.model == kBsnq;
     const int friction = A.phy.friction;
@@ -675,7 +714,6 @@ __device__ __forceinline__ void stencil_tile_pair(const StencilArgs<float> &A, c
 
     if (rows > 0) {
     pk qn[3], hi[3], Hs[3], dhi;   // row r + 1; cell r's values at its north face; flux through its south face
-    DiffRow below;                 // x-differences of row r - 1
     pk dS;                         // depth d of row r - 1
     {
         const pk q2[3] = {ldp(pw - 2 * kPS), ldp(pQ - 2 * kPQ), ldp(pw + oP - 2 * kPS)};
@@ -691,11 +729,8 @@ __device__ __forceinline__ void stencil_tile_pair(const StencilArgs<float> &A, c
         fix_pair(q1[0], mul2(hlf, cm.h), mul2(hlf, c0.h), lo[0], hm[0], dl, dm);
         recon_pair(A, q1, q, qn, mul2(hlf, c0.h), mul2(hlf, c1.h), lo, hi, dl, dhi);
         fix_pair(q[0], mul2(hlf, c0.h), mul2(hlf, c1.h), lo[0], hi[0], dl, dhi);
-        flux_pair<false>(A, hm, dm, lo, dl, Hs);
-        if (bsnq) {
-            below = diff_row(side_row(pw - kPS, pw + oP - kPS, pQ - kPQ), q1[0], q1[2], q1[1]);
-            dS = depth_pair(A, bbar_pair(A, cm, c0));
-        }
+        flux_v<pk>(A, hm, dm, lo, dl, Hs);
+        if (bsnq) dS = depth_pair(A, bbar_pair(A, cm, c0));
     }
 #pragma unroll 1
     for (int r = 0; r < rows; r++) {
@@ -718,8 +753,7 @@ __device__ __forceinline__ void stencil_tile_pair(const StencilArgs<float> &A, c
             const pk qq[3] = {ldp(pw + 2 * kPS), ldp(pQ + 2 * kPQ), ldp(pw + oP + 2 * kPS)};
             recon_pair(A, q, qn, qq, By0, By1, ly, hy, dly, dhy);
         }
-        DiffRow here;
-        pk w3, Bx0, Bx1, sx;                 // w(x + 2) - w(x - 2); face beds; their sums' differences
+        pk Bx0, Bx1, sx;                     // face beds; their sums' differences
         {
             const SideRow side = side_row(pw, pw + oP, pQ);
             float a, b, v0, v1;
@@ -742,40 +776,41 @@ __device__ __forceinline__ void stencil_tile_pair(const StencilArgs<float> &A, c
             qm[2] = mk(side.ql, a);
             q0[2] = q[1];
             qp[2] = mk(b, side.qr);
-            here.w = sub2(qp[0], qm[0]);
-            here.ww = sub2(sub2(qp[0], q[0]), sub2(q[0], qm[0]));
-            here.P = sub2(qp[1], qm[1]);
-            here.Q = sub2(qp[2], qm[2]);
-            w3 = sub2(mk(side.wr, side.wrr), mk(side.wll, side.wl));
             recon_pair(A, qm, q0, qp, Bx0, Bx1, lx, hx, dlx, dhx);
         }
         const pk Bb = bbar_pair(A, c0, c1), sy = sub2(c1.h, c0.h), hb = sub2(q[0], Bb);
-        // Fluxes through the north faces and the west faces, and friction:
-        // one branch for the row, on whether every depth reaches eps^(1/4)
-        // (then no fix is due, and a cell's own depth, the mean of its
-        // faces', reaches it too).
-        pk Hn[3], H[3], fr = 0;
-        const float thin = fminf(fminf(least(dly, dhy), least(dlx, dhx)), fminf(px_(dhi), py_(dhi)));
-        if (__all_sync(0xffffffffu, thin >= C.hwet)) {
-            const pk Lx[3] = {from_left(hx[0]), from_left(hx[1]), from_left(hx[2])};
-            const pk dL = from_left(dhx);
-            flux_pair<true>(A, hi, dhi, ly, dly, Hn);
-            flux_pair<true>(A, Lx, dL, lx, dlx, H);
-            if (friction != kFricNone) fr = friction_pair<true>(A, friction, hb, q[2], q[1]);
-        } else {
+        // Fluxes through the north faces and the west faces, and friction.
+        // One branch for the row: the fix changes nothing where no depth is
+        // negative.  Only faces of the grid's cells count (along x also those
+        // of cell nx, whose low side the last face takes), not what lies
+        // unwritten beyond them.
+        pk Hn[3], H[3];
+        float y0m, y1m, x0m, x1m;
+        {
+            float a, b;
+            un(dly, y0m, y1m);
+            un(dhy, a, b);
+            y0m = fminf(y0m, a);
+            y1m = fminf(y1m, b);
+            un(dlx, x0m, x1m);
+            un(dhx, a, b);
+            x0m = fminf(x0m, a);
+            x1m = fminf(x1m, b);
+        }
+        if (__any_sync(0xffffffffu, (ok0 && (y0m < 0.f || x1m < 0.f)) || (ok1 && y1m < 0.f) || (i <= nx && x0m < 0.f))) {
             fix_pair(qn[0], By0, By1, ly[0], hy[0], dly, dhy);
             fix_pair(q[0], Bx0, Bx1, lx[0], hx[0], dlx, dhx);
-            const pk Lx[3] = {from_left(hx[0]), from_left(hx[1]), from_left(hx[2])};
-            const pk dL = from_left(dhx);
-            flux_pair<false>(A, hi, dhi, ly, dly, Hn);
-            flux_pair<false>(A, Lx, dL, lx, dlx, H);
-            if (friction != kFricNone) fr = friction_pair<false>(A, friction, hb, q[2], q[1]);
         }
-        CarryPair cw, cu, cv;
+        {
+            const pk Lx[3] = {from_left(hx[0]), from_left(hx[1]), from_left(hx[2])};
+            flux_v<pk>(A, hi, dhi, ly, dly, Hn);
+            flux_v<pk>(A, Lx, from_left(dhx), lx, dlx, H);
+        }
+        CarryV<pk> cw, cu, cv;
         if (kSpec == 2 && ok0) {
-            cw = load_carry_pair<kSpec>(A, 0, kr);
-            cu = load_carry_pair<kSpec>(A, 1, kr);
-            cv = load_carry_pair<kSpec>(A, 2, kr);
+            cw = load_carry_v<pk, kSpec>(A, 0, kr);
+            cu = load_carry_v<pk, kSpec>(A, 1, kr);
+            cv = load_carry_v<pk, kSpec>(A, 2, kr);
         }
         // flux differences: south less north, west less east (the next lane's
         // west face; the tile's edge faces from the first pass)
@@ -808,51 +843,38 @@ __device__ __forceinline__ void stencil_tile_pair(const StencilArgs<float> &A, c
         const pk uu = ldv(pw + 2 * kPS);
         // the history this stage reads (asked into L2 at the tile's start)
         if (kSpec != 2 && ok0) {
-            cw = load_carry_pair<kSpec>(A, 0, kr);
-            cu = load_carry_pair<kSpec>(A, 1, kr);
-            cv = load_carry_pair<kSpec>(A, 2, kr);
+            cw = load_carry_v<pk, kSpec>(A, 0, kr);
+            cu = load_carry_v<pk, kSpec>(A, 1, kr);
+            cv = load_carry_v<pk, kSpec>(A, 2, kr);
         }
         // right sides: bed slope (half the corner sums' differences), friction, dispersion
         const pk dd = depth_pair(A, Bb);
-        pk F = fma2(fr, u[2], fma2(mul2(hb, kc(A, kcMHgx)), sx, dv[1]));
-        pk Gq = fma2(fr, u[1], fma2(mul2(hb, kc(A, kcMHgy)), sy, dv[2]));
+        const pk gh = mul2(kc(A, kcMHalfG), hb);
+        pk F = fma2(mul2(gh, sx), kc(A, kcRdx), dv[1]);
+        pk Gq = fma2(mul2(gh, sy), kc(A, kcRdy), dv[2]);
+        if (friction != kFricNone) friction_v<pk>(A, friction, hb, u[2], u[1], F, Gq);
         pk Fs = 0, Gs = 0;
         if (bsnq) {
             const pk dN = depth_pair(A, bbar_pair(A, e1, e2));
-            const DiffRow above = diff_row(side_row(pw + kPS, pw + oP + kPS, pQ + kPQ), cn[0], cn[2], cn[1]);
-            const pk wS = ldp(pw - kPS), wSS = ldp(pw - 2 * kPS), PS = ldp(pw + oP - kPS), QS = ldp(pQ - kPQ);
             float a, b;
             un(dd, a, b);
             float dl = __shfl_up_sync(0xffffffffu, b, 1), dr = __shfl_down_sync(0xffffffffu, a, 1);
             if (atW) dl = pe[r].w;
             if (atE) dr = pe[r].w;
-            const pk dDx = mk(b - dl, dr - a), dDy = sub2(dN, dS);
-            const pk two = kc(A, kcTwo), mtwo = kc(A, kcMTwo);
-            const pk gy = sub2(cn[0], wS);
-            const pk eyy = sub2(sub2(cn[0], u[0]), sub2(u[0], wS));
-            const pk eyyy = fma2(mtwo, gy, sub2(uu, wSS));
-            const pk exxx = fma2(mtwo, here.w, w3);
-            const pk exy = mul2(kc(A, kcQ), sub2(above.w, below.w));
-            const pk exyy = fma2(mtwo, here.w, add2(above.w, below.w));
-            const pk exxy = sub2(above.ww, below.ww);
-            // K d^2 / (2 dx) [A (d exxx + 2 d_x exx) + B (d exyy + d_x eyy + d_y exy / 4)], A = 1/dx^2, B = 1/dy^2
-            const pk d2 = mul2(dd, dd), Ax = kc(A, kcRdx2), By = kc(A, kcRdy2);
-            const pk x1 = fma2(mul2(two, dDx), here.ww, mul2(dd, exxx));
-            const pk x2 = fma2(dDy, exy, fma2(dDx, eyy, mul2(dd, exyy)));
-            const pk y1 = fma2(mul2(two, dDy), eyy, mul2(dd, eyyy));
-            const pk y2 = fma2(dDx, exy, fma2(dDy, here.ww, mul2(dd, exxy)));
-            F = fma2(mul2(d2, kc(A, kcKx)), fma2(By, x2, mul2(Ax, x1)), F);
-            Gq = fma2(mul2(d2, kc(A, kcKy)), fma2(Ax, y2, mul2(By, y1)), Gq);
-            const pk dc = mul2(dd, kc(A, kcC6)), m1 = mul2(dc, dDx), m2 = mul2(dc, dDy), m3 = mul2(d2, kc(A, kcB3xy));
-            Fs = fma2(m3, sub2(above.Q, below.Q), fma2(m2, here.Q, mul2(m1, sub2(cn[1], QS))));
-            Gs = fma2(m3, sub2(above.P, below.P), fma2(m1, sub2(cn[2], PS), mul2(m2, here.P)));
+            const pk ddx = mul2(mk(b - dl, dr - a), kc(A, kcHrdx)), ddy = mul2(sub2(dN, dS), kc(A, kcHrdy));
+            Around<pk> e = aroundv<kPS>(pw, u[0], cn[0], ldv(pw - kPS));
+            e.nn = uu;
+            e.ss = ldv(pw - 2 * kPS);
+            eta_terms_v(A, e, dd, ddx, ddy, F, Gq);
+            Fs = mixed_term_v(A, aroundv<kPQ>(pQ, u[1], cn[1], ldv(pQ - kPQ)), dd, ddx, ddy);
+            Gs = mixed_term_v(A, aroundv<kPS>(pw + oP, u[2], cn[2], ldv(pw + oP - kPS)), dd, ddx, ddy);
         }
         // update
-        const pk dw = advance_pair<kSpec>(A, 0, u[0], dv[0], 0, kr, cw, ok0);
-        const pk dU = advance_pair<kSpec>(A, 1, 0, F, Fs, kr, cu, ok0);
-        const pk dV = advance_pair<kSpec>(A, 2, 0, Gq, Gs, kr, cv, ok0);
+        const pk dw = advance_v<pk, kSpec>(A, 0, u[0], dv[0], 0, kr, cw, ok0);
+        const pk dU = advance_v<pk, kSpec>(A, 1, 0, F, Fs, kr, cu, ok0);
+        const pk dV = advance_v<pk, kSpec>(A, 2, 0, Gq, Gs, kr, cv, ok0);
         float a, b, B0, B1;
-        un(kSpec == 2 ? dw : add2(u[0], dw), a, b);   // the AM4 base of w holds w^n
+        un(kSpec != 0 ? dw : add2(u[0], dw), a, b);
         un(Bb, B0, B1);
         if (a < B0) a = B0;                  // Reading A-D1
         if (b < B1) b = B1;
@@ -892,7 +914,6 @@ __device__ __forceinline__ void stencil_tile_pair(const StencilArgs<float> &A, c
             qn[1] = ldv(pQ + 2 * kPQ);
             qn[2] = ldv(pw + oP + 2 * kPS);
         }
-        below = here;
         dS = dd;
         pw += kPS;
         pQ += kPQ;
