@@ -309,7 +309,7 @@ __device__ __forceinline__ void face_flux_vjp(const T w[4], const T P[4], const 
     const bool apK = not_below(ap1), amK = !above_zero(am1);
     const T ap = apK ? ap1 : T(0), am = amK ? am1 : T(0);
     const T den = ap - am;
-    if (!above_zero(den)) return;
+    if (is_zero(den)) return;
     const T inv = rcp_r(den), apam = ap * am;
     const T FL1 = qnL * uL + T(0.5) * (ghL * hL), FR1 = qnR * uR + T(0.5) * (ghR * hR);
     const T FL2 = qnL * vL, FR2 = qnR * vR;

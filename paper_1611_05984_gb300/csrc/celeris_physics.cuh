@@ -171,7 +171,10 @@ __device__ __forceinline__ bool below_zero(double x)
     const unsigned hi = (unsigned)__double2hiint(x);
     return hi - 0x80000000u < 0x7ff00001u && (hi << 1 | (unsigned)__double2loint(x)) != 0u;
 }
-// x > 0, and x >= y for y > 0 (FP64: as integers)
+// x == 0 (false for NaN)
+__device__ __forceinline__ bool is_zero(float x) { return x == 0.f; }
+__device__ __forceinline__ bool is_zero(double x) { return (__double_as_longlong(x) << 1) == 0; }
+// x > 0, and x >= y for y > 0 (FP64: as integers, a NaN by its sign)
 __device__ __forceinline__ bool above_zero(float x) { return x > 0.f; }
 __device__ __forceinline__ bool above_zero(double x) { return __double_as_longlong(x) > 0; }
 __device__ __forceinline__ bool at_least(float x, float y) { return x >= y; }
@@ -186,7 +189,8 @@ __device__ __forceinline__ long long order_key(double x)
     const long long k = __double_as_longlong(x);
     return k ^ ((k >> 63) & 0x7fffffffffffffffll);
 }
-// max(a, b, 0) and min(a, b, 0)
+// max(a, b, 0) and min(a, b, 0) (FP64: a NaN ranks beyond the infinity of its
+// sign, so that of two speeds' extremes one is it)
 __device__ __forceinline__ float max_zero(float a, float b)
 {
     float d;
@@ -317,12 +321,11 @@ struct FaceSweep {
 
 // KP07 step 3: the central-upwind flux H = (mass, normal, tangential
 // momentum) from the face values (w, normal, tangential discharge) and depths.
-template <typename real>
-__device__ __forceinline__ void face_flux_step(real g, real eps, real hwet, real wL, real nL, real tL, real hL, real wR,
-                                               real nR, real tR, real hR, real H[3])
+__device__ __forceinline__ void face_flux_step(double g, double eps, double hwet, double wL, double nL, double tL,
+                                               double hL, double wR, double nR, double tR, double hR, double H[3])
 {
-    const real ghL = mul_r(g, hL), ghR = mul_r(g, hR);
-    real sL, sR, kL, kR;
+    const double ghL = mul_r(g, hL), ghR = mul_r(g, hR);
+    double sL, sR, kL, kR;
     const bool wet = at_least(hL, hwet) && at_least(hR, hwet);
     if (wet) {
         root_and_inverse(g, hL, ghL, sL, kL);
@@ -333,25 +336,25 @@ __device__ __forceinline__ void face_flux_step(real g, real eps, real hwet, real
         sL = sqrt_r(ghL);
         sR = sqrt_r(ghR);
     }
-    const real uL = mul_r(kL, nL), vL = mul_r(kL, tL), uR = mul_r(kR, nR), vR = mul_r(kR, tR);
+    const double uL = mul_r(kL, nL), vL = mul_r(kL, tL), uR = mul_r(kR, nR), vR = mul_r(kR, tR);
     if (!wet) {
         nL = mul_r(hL, uL);
         tL = mul_r(hL, vL);
         nR = mul_r(hR, uR);
         tR = mul_r(hR, vR);
     }
-    const real ap = max_zero(add_r(uL, sL), add_r(uR, sR));
-    const real am = min_zero(sub_r(uL, sL), sub_r(uR, sR));
-    const real den = sub_r(ap, am);
-    if (!above_zero(den)) {   // both sides dry (Reading A-F1)
-        H[0] = H[1] = H[2] = real(0);
+    const double ap = max_zero(add_r(uL, sL), add_r(uR, sR));
+    const double am = min_zero(sub_r(uL, sL), sub_r(uR, sR));
+    const double den = sub_r(ap, am);
+    if (is_zero(den)) {   // both sides dry (Reading A-F1); a NaN goes on into the flux
+        H[0] = H[1] = H[2] = 0.0;
         return;
     }
     // (a+ F_L - a- F_R + a+ a- (q_R - q_L)) / (a+ - a-) = F_L + beta (F_R - F_L) - a+ beta (q_R - q_L), beta = -a-/(a+ - a-)
-    const real beta = mul_r(-am, rcp_r(den)), nab = mul_r(-ap, beta);
-    const real FL1 = fma(real(0.5), mul_r(ghL, hL), mul_r(nL, uL)), FR1 = fma(real(0.5), mul_r(ghR, hR), mul_r(nR, uR));
-    const real FL2 = mul_r(nL, vL);
-    const real dn = sub_r(nR, nL);
+    const double beta = mul_r(-am, rcp_r(den)), nab = mul_r(-ap, beta);
+    const double FL1 = fma(0.5, mul_r(ghL, hL), mul_r(nL, uL)), FR1 = fma(0.5, mul_r(ghR, hR), mul_r(nR, uR));
+    const double FL2 = mul_r(nL, vL);
+    const double dn = sub_r(nR, nL);
     H[0] = fma(nab, sub_r(wR, wL), fma(beta, dn, nL));
     H[1] = fma(nab, dn, fma(beta, sub_r(FR1, FL1), FL1));
     H[2] = fma(nab, sub_r(tR, tL), fma(beta, fma(nR, vR, -FL2), FL2));
