@@ -290,6 +290,15 @@ cel_status cel_adjoint_input_gradient(cel_solver *s, const void *w_in_dev, void 
 cel_status cel_adjoint_face_selfcheck(int32_t real_bytes, const void *in_dev, int32_t n, void *out_dev,
                                       void *cuda_stream);
 
+/* Self-check of the double-precision step's own elementary functions: op of
+ * n values, out[k] = op(in[k]).  CEL_OP_RECIPROCAL: 1/x, normal x of normal
+ * 1/x.  CEL_OP_SQRT: every x.  CEL_OP_RCBRT: x^(-1/3), x from 2^-126 to 2^127.
+ * CEL_OP_HALF: x/2, |x| below 2^-1021 unchanged.  in_dev, out_dev: [n]
+ * double, device.  cuda_stream as in cel_create.  Synchronises; CEL_ERR_CUDA
+ * on a CUDA error, CEL_ERR_INVALID_ARG on bad arguments. */
+typedef enum { CEL_OP_RECIPROCAL = 0, CEL_OP_SQRT = 1, CEL_OP_RCBRT = 2, CEL_OP_HALF = 3 } cel_arithmetic_op;
+cel_status cel_arithmetic_selfcheck(int32_t op, const void *in_dev, int32_t n, void *out_dev, void *cuda_stream);
+
 /* Line-solver splits (the per-line tridiagonal solves of Eq. 21-23).  A
  * line of up to 8192 rows (FP32) or 4096 (FP64) is cut into segments of 2, 4
  * or 8 rows, one per thread: the built-in rule takes 2 rows on lines of at

@@ -33,6 +33,7 @@ EXPORTS = ["cel_workspace_bytes", "cel_create", "cel_set_boundary", "cel_set_sta
            "cel_check_finite", "cel_checkpoint_bytes", "cel_save_checkpoint",
            "cel_load_checkpoint", "cel_runup_enable", "cel_render", "cel_adjoint_bytes",
            "cel_adjoint_gauge_misfit", "cel_adjoint_face_selfcheck", "cel_adjoint_input_gradient",
+           "cel_arithmetic_selfcheck",
            "cel_get_stats", "cel_last_launch_count", "cel_profile_enable",
            "cel_profile_read", "cel_profile_disable", "cel_ensemble_table_bytes",
            "cel_ensemble_create", "cel_ensemble_step", "cel_ensemble_use_graphs", "cel_ensemble_graph_steps",
@@ -111,6 +112,7 @@ def load(build_if_missing: bool = True):
         L.cel_adjoint_gauge_misfit.argtypes = [vp, i32, i32, ctypes.POINTER(i32), i32, vp, vp, sz, vp, vp, vp,
                                                ctypes.POINTER(d)]
         L.cel_adjoint_face_selfcheck.argtypes = [i32, vp, i32, vp, vp]
+        L.cel_arithmetic_selfcheck.argtypes = [i32, vp, i32, vp, vp]
         L.cel_adjoint_input_gradient.argtypes = [vp, vp, vp]
         L.cel_get_stats.argtypes = [vp, ctypes.POINTER(CelStats)]
         L.cel_last_launch_count.argtypes = [vp, ctypes.POINTER(i64)]
@@ -632,6 +634,21 @@ def face_vjp_selfcheck(inputs):
     if st != 0:
         raise CelerisError(f"face_vjp_selfcheck failed ({st})")
     return out[:, :15], out[:, 15:]
+
+
+def arithmetic_selfcheck(op: str, x):
+    """The double-precision step's own "reciprocal", "sqrt", "rcbrt" or "half"
+    of the values in `x`, a float64 CUDA tensor (cel_arithmetic_selfcheck)."""
+    import torch
+    x = x.contiguous()
+    if x.dtype != torch.float64 or not x.is_cuda:
+        raise ValueError("x must be a float64 CUDA tensor")
+    out = torch.empty_like(x)
+    st = load().cel_arithmetic_selfcheck(["reciprocal", "sqrt", "rcbrt", "half"].index(op), x.data_ptr(), x.numel(),
+                                         out.data_ptr(), torch.cuda.current_stream(x.device).cuda_stream)
+    if st != 0:
+        raise CelerisError(f"arithmetic_selfcheck failed ({st})")
+    return out
 
 
 def _gauge_misfit_function():

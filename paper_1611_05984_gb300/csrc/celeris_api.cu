@@ -2622,6 +2622,16 @@ cel_status cel_adjoint_face_selfcheck(int32_t real_bytes, const void *in_dev, in
     return e == cudaSuccess ? CEL_OK : CEL_ERR_CUDA;
 }
 
+cel_status cel_arithmetic_selfcheck(int32_t op, const void *in_dev, int32_t n, void *out_dev, void *cuda_stream)
+{
+    if (op < CEL_OP_RECIPROCAL || op > CEL_OP_HALF || n < 0 || (n > 0 && (!in_dev || !out_dev))) return CEL_ERR_INVALID_ARG;
+    if (n == 0) return CEL_OK;
+    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    cudaError_t e = launch_arithmetic_check(op, (const double *)in_dev, n, (double *)out_dev, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    return e == cudaSuccess ? CEL_OK : CEL_ERR_CUDA;
+}
+
 cel_status cel_adjoint_bytes(const cel_solver *s, int32_t nsteps, int32_t ckpt_every, int32_t ngauges,
                              int32_t with_bed, size_t *bytes)
 {

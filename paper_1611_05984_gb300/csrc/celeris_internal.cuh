@@ -451,6 +451,9 @@ struct PersistArgs {
     int barrier_only;                  // 1: one barrier and nothing else (a check of the waits' bound)
 };
 
+// The FP64 kernels' own elementary functions (cel_arithmetic_selfcheck).
+cudaError_t launch_arithmetic_check(int op, const double *in, int n, double *out, cudaStream_t st);
+
 // k: the lockstep step index, plus *kdev where kdev is given (a device
 // counter that a captured graph advances between its replays).
 template <typename real>

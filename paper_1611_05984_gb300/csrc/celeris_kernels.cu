@@ -2313,7 +2313,21 @@ cudaError_t launch_ghost_batch(const GhostArgs<real> *args, const int *start, in
 
 namespace {
 __global__ void k_counter(int64_t *p, int64_t v, int add) { *p = add ? *p + v : v; }
+
+__global__ void k_arithmetic_check(int op, const double *in, int n, double *out)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    const double x = in[k];
+    out[k] = op == CEL_OP_RECIPROCAL ? rcp_r(x) : op == CEL_OP_SQRT ? sqrt_r(x) : op == CEL_OP_RCBRT ? rcbrt_r(x) : half_r(x);
+}
 }  // namespace
+
+cudaError_t launch_arithmetic_check(int op, const double *in, int n, double *out, cudaStream_t st)
+{
+    k_arithmetic_check<<<(n + 127) / 128, 128, 0, st>>>(op, in, n, out);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_counter(int64_t *p, int64_t v, int add, cudaStream_t st)
 {

@@ -155,13 +155,14 @@ __device__ __forceinline__ void root_and_inverse(double g, double h, double gh, 
     ih = mul_r(mul_r(g, r), r);
 }
 
-// x / 2 (FP64: on the exponent; values below 2^-1021 as they are, which
-// changes a sum by less than that).
+// x / 2 (FP64: on the exponent; infinities and NaN as they are, and values
+// below 2^-1021, which changes a sum by less than that).
 __device__ __forceinline__ float half_r(float x) { return 0.5f * x; }
 __device__ __forceinline__ double half_r(double x)
 {
     const int hi = __double2hiint(x);
-    return __hiloint2double((hi & 0x7ff00000) > 0x00100000 ? hi - 0x00100000 : hi, __double2loint(x));
+    const bool scale = (unsigned)(hi & 0x7ff00000) - 0x00200000u < 0x7fd00000u;   // exponent field 2 .. 0x7fe
+    return __hiloint2double(scale ? hi - 0x00100000 : hi, __double2loint(x));
 }
 
 // x < 0 (false for NaN and -0)

@@ -112,6 +112,16 @@ def test_adjoint_entry_points_reject_bad_arguments_without_gpu_work():
     assert L.cel_adjoint_face_selfcheck(4, None, 0, None, None) == 0     # nothing to do
 
 
+def test_arithmetic_selfcheck_rejects_bad_arguments_without_gpu_work():
+    """An unknown operation, a negative count, NULL buffers; nothing to do."""
+    L = celeris.load()
+    assert L.cel_arithmetic_selfcheck(-1, None, 4, None, None) == 1
+    assert L.cel_arithmetic_selfcheck(4, None, 4, None, None) == 1
+    assert L.cel_arithmetic_selfcheck(0, None, -1, None, None) == 1
+    assert L.cel_arithmetic_selfcheck(0, None, 5, None, None) == 1
+    assert L.cel_arithmetic_selfcheck(3, None, 0, None, None) == 0
+
+
 def test_line_split_table():
     """The line solver's split per class of line lengths (cel_set_line_split,
     the autotuner's setting): the built-in rule, a class overriding it where

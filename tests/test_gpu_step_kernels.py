@@ -187,3 +187,34 @@ def test_single_precision_bits(case, crc):
     fields = [a.cpu().numpy() for a in g.state()]
     assert all(np.isfinite(a).all() for a in fields)
     assert [zlib.crc32((a + np.float32(0)).tobytes()) for a in fields] == list(crc)   # -0 as 0
+
+
+def _spread(lo, hi, n=200000):
+    """Positive doubles of every exponent from 2^lo to 2^hi, the ends among them."""
+    rng = np.random.default_rng(11)
+    x = np.ldexp(rng.uniform(1.0, 2.0, n), rng.integers(lo, hi, n))
+    return np.concatenate([x, [2.0 ** lo, 2.0 ** hi], np.ldexp(1.0, np.arange(lo, hi, max(1, (hi - lo) // 500)))])
+
+
+# largest errors in units of the result's last place: the reciprocal's last
+# operation rounds once and its remainder is e^3 with e < 2^-20; x^(-1/3) adds two
+# roundings in e = 1 - x r^3, a third of each
+@pytest.mark.parametrize("op,lo,hi,ulp", [("reciprocal", -1021, 1021, 0.51), ("rcbrt", -126, 127, 1.7)])
+def test_fp64_elementary_functions(op, lo, hi, ulp):
+    """The FP64 kernels' own functions over the exponents they serve, against
+    extended precision."""
+    from paper_1611_05984_gb300 import celeris
+    x = _spread(lo, hi)
+    wide = x.astype(np.longdouble)
+    ref = {"reciprocal": lambda: 1 / wide, "rcbrt": lambda: 1 / np.cbrt(wide)}[op]()
+    got = celeris.arithmetic_selfcheck(op, torch.from_numpy(x).cuda()).cpu().numpy()
+    err = (np.abs(got.astype(np.longdouble) - ref) / np.spacing(ref.astype(np.float64))).astype(np.float64)
+    assert err.max() <= ulp, (err.max(), x[err.argmax()])
+
+
+def test_fp64_half_keeps_what_is_not_finite():
+    from paper_1611_05984_gb300 import celeris
+    x = np.concatenate([_spread(-1021, 1023), [0.0, np.inf, np.nan, np.finfo(np.float64).max, 5e-324, 2.0 ** -1022]])
+    x = np.concatenate([x, -x])
+    got = celeris.arithmetic_selfcheck("half", torch.from_numpy(x).cuda()).cpu().numpy()
+    np.testing.assert_array_equal(got, np.where(np.abs(x) < 2.0 ** -1021, x, 0.5 * x))
