@@ -279,20 +279,16 @@ __device__ __forceinline__ void face_flux_vjp(const T w[4], const T P[4], const 
     // factor is 1/h there); cL, cR: d(celerity)/dh
     const bool wet = at_least(hL, hwet) && at_least(hR, hwet);
     const T ghL = g * hL, ghR = g * hR;
-    T kL, kR, sL, sR, cL, cR, qnL = nL, qtL = tL, qnR = nR, qtR = tR;
+    const T sL = sqrt_r(ghL), sR = sqrt_r(ghR);
+    T kL, kR, cL, cR, qnL = nL, qtL = tL, qnR = nR, qtR = tR;
     if (wet) {
-        const T rL = rsqrt_r(ghL), rR = rsqrt_r(ghR);
-        sL = ghL * rL;
-        sR = ghR * rR;
-        kL = g * rL * rL;
-        kR = g * rR * rR;
-        cL = T(0.5) * g * rL;
-        cR = T(0.5) * g * rR;
+        kL = rcp_r(hL);
+        kR = rcp_r(hR);
+        cL = half_r(g) * rcp_r(sL);
+        cR = half_r(g) * rcp_r(sR);
     } else {
         kL = desing(hL, eps);
         kR = desing(hR, eps);
-        sL = sqrt(ghL);
-        sR = sqrt(ghR);
         cL = sL > T(0) ? g / (T(2) * sL) : T(0);
         cR = sR > T(0) ? g / (T(2) * sR) : T(0);
     }

@@ -97,8 +97,8 @@ __device__ __forceinline__ void cu_flux(real g, real eps, real wL, real nL, real
 // In FP64 every add, multiply and comparison runs on a pipe of two lanes per
 // SM, which bounds the FP64 stencil, so comparisons, maxima and halvings work
 // on the bit patterns with integer instructions, and reciprocals and roots are
-// refined from the hardware's approximations by one third-order step
-// (Householder's method).  2048 x 2048 beach, both stages and the line solves
+// refined from the hardware's approximations (Householder's third-order step;
+// Goldschmidt's iteration and a remainder).  2048 x 2048 beach, both stages and the line solves
 // of 2 Euler and 2 full steps: 27.4 ms before, 20.0 ms with these forms (the
 // stencil's FP64 instructions per cell from about 580 to 350).
 
@@ -127,34 +127,6 @@ __device__ __forceinline__ double rcp_r(double x)
     const double e = fma(-x, y, 1.0);
     return fma(y, fma(e, e, e), y);
 }
-// 1/sqrt(x) for normal x > 0: y(1 + e/2 + 3 e^2/8) with e = 1 - x y^2.
-__device__ __forceinline__ double rsqrt_r(double x)
-{
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(mul_r(-x, y), y, 1.0);
-    return fma(mul_r(fma(0.375, e, 0.5), e), y, y);
-}
-
-__device__ __forceinline__ float sqrt_r(float x) { return sqrtf(x); }
-__device__ __forceinline__ double sqrt_r(double x)
-{
-    // near the ends of the range (subnormals and infinity among them) the plain root
-    if ((unsigned)__double2hiint(x) - 0x01700000u < 0x7e800000u) return mul_r(x, rsqrt_r(x));
-    return __double_as_longlong(x) == 0 ? 0.0 : sqrt(x);
-}
-
-// 1 / sqrt(x)
-__device__ __forceinline__ float rsqrt_r(float x) { return rsqrtf(x); }
-
-// sqrt(x) and c / x' for x = g h, c = g: the celerity and 1/h from one root.
-__device__ __forceinline__ void root_and_inverse(double g, double h, double gh, double &s, double &ih)
-{
-    const double r = rsqrt_r(gh);
-    s = mul_r(gh, r);
-    ih = mul_r(mul_r(g, r), r);
-}
-
 // x / 2 (FP64: on the exponent; infinities and NaN as they are, and values
 // below 2^-1021, which changes a sum by less than that).
 __device__ __forceinline__ float half_r(float x) { return 0.5f * x; }
@@ -163,6 +135,23 @@ __device__ __forceinline__ double half_r(double x)
     const int hi = __double2hiint(x);
     const bool scale = (unsigned)(hi & 0x7ff00000) - 0x00200000u < 0x7fd00000u;   // exponent field 2 .. 0x7fe
     return __hiloint2double(scale ? hi - 0x00100000 : hi, __double2loint(x));
+}
+
+__device__ __forceinline__ float sqrt_r(float x) { return sqrtf(x); }
+// sqrt(x): from y = 1/sqrt(x) (1 + e) one Goldschmidt step on s = x y and h = y/2
+// (both 1 + O(e^2) off), then s + h (x - s^2) with the remainder exact to one
+// rounding: what is left is s's own rounding (0.5001 units of the last place).
+__device__ __forceinline__ double sqrt_r(double x)
+{
+    // near the ends of the range (subnormals and infinity among them) the plain root
+    if ((unsigned)__double2hiint(x) - 0x01700000u < 0x7e800000u) {
+        double y;
+        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+        const double s0 = mul_r(x, y), h0 = half_r(y), r = fma(-s0, h0, 0.5);
+        const double s = fma(s0, r, s0), h = fma(h0, r, h0);
+        return fma(fma(-s, s, x), h, s);
+    }
+    return __double_as_longlong(x) == 0 ? 0.0 : sqrt(x);
 }
 
 // x < 0 (false for NaN and -0)
@@ -326,17 +315,9 @@ __device__ __forceinline__ void face_flux_step(double g, double eps, double hwet
                                                double hL, double wR, double nR, double tR, double hR, double H[3])
 {
     const double ghL = mul_r(g, hL), ghR = mul_r(g, hR);
-    double sL, sR, kL, kR;
+    const double sL = sqrt_r(ghL), sR = sqrt_r(ghR);
     const bool wet = at_least(hL, hwet) && at_least(hR, hwet);
-    if (wet) {
-        root_and_inverse(g, hL, ghL, sL, kL);
-        root_and_inverse(g, hR, ghR, sR, kR);
-    } else {
-        kL = desing(hL, eps);
-        kR = desing(hR, eps);
-        sL = sqrt_r(ghL);
-        sR = sqrt_r(ghR);
-    }
+    const double kL = wet ? rcp_r(hL) : desing(hL, eps), kR = wet ? rcp_r(hR) : desing(hR, eps);
     const double uL = mul_r(kL, nL), vL = mul_r(kL, tL), uR = mul_r(kR, nR), vR = mul_r(kR, tR);
     if (!wet) {
         nL = mul_r(hL, uL);

@@ -196,20 +196,28 @@ def _spread(lo, hi, n=200000):
     return np.concatenate([x, [2.0 ** lo, 2.0 ** hi], np.ldexp(1.0, np.arange(lo, hi, max(1, (hi - lo) // 500)))])
 
 
-# largest errors in units of the result's last place: the reciprocal's last
-# operation rounds once and its remainder is e^3 with e < 2^-20; x^(-1/3) adds two
-# roundings in e = 1 - x r^3, a third of each
-@pytest.mark.parametrize("op,lo,hi,ulp", [("reciprocal", -1021, 1021, 0.51), ("rcbrt", -126, 127, 1.7)])
+# largest errors in units of the result's last place: the last operation of the
+# reciprocal and of the root rounds once, and their remainders are e^3 and e^4 with
+# e < 2^-20; x^(-1/3) adds two roundings in e = 1 - x r^3, a third of each
+@pytest.mark.parametrize("op,lo,hi,ulp", [("reciprocal", -1021, 1021, 0.51), ("sqrt", -1074, 1023, 0.51),
+                                          ("rcbrt", -126, 127, 1.7)])
 def test_fp64_elementary_functions(op, lo, hi, ulp):
     """The FP64 kernels' own functions over the exponents they serve, against
     extended precision."""
     from paper_1611_05984_gb300 import celeris
     x = _spread(lo, hi)
     wide = x.astype(np.longdouble)
-    ref = {"reciprocal": lambda: 1 / wide, "rcbrt": lambda: 1 / np.cbrt(wide)}[op]()
+    ref = {"reciprocal": lambda: 1 / wide, "sqrt": lambda: np.sqrt(wide), "rcbrt": lambda: 1 / np.cbrt(wide)}[op]()
     got = celeris.arithmetic_selfcheck(op, torch.from_numpy(x).cuda()).cpu().numpy()
     err = (np.abs(got.astype(np.longdouble) - ref) / np.spacing(ref.astype(np.float64))).astype(np.float64)
     assert err.max() <= ulp, (err.max(), x[err.argmax()])
+
+
+def test_fp64_root_at_the_ends():
+    from paper_1611_05984_gb300 import celeris
+    x = np.array([0.0, -0.0, np.inf, np.nan, -1.0, -np.inf])
+    got = celeris.arithmetic_selfcheck("sqrt", torch.from_numpy(x).cuda()).cpu().numpy()
+    np.testing.assert_array_equal(got, [0.0, 0.0, np.inf, np.nan, np.nan, np.nan])
 
 
 def test_fp64_half_keeps_what_is_not_finite():
