@@ -344,8 +344,10 @@ __device__ __forceinline__ void face_flux_step(double g, double eps, double hwet
 
 __device__ __forceinline__ float cbrt_r(float x) { return x > 0.f ? exp2f(__log2f(x) * (1.f / 3.f)) : 0.f; }
 __device__ __forceinline__ double cbrt_r(double x) { return cbrt(x); }
-// h^(-1/3) for normal h > 0 in the range of single precision: one
-// third-order step r(1 + e/3 + 2 e^2/9), e = 1 - h r^3, from a single-precision value.
+// 2^-126 <= h < 2^127: normal in single precision, and so is its reciprocal
+__device__ __forceinline__ bool in_single_range(double h) { return (unsigned)__double2hiint(h) - 0x38100000u < 0x0fd00000u; }
+// h^(-1/3) for h in that range: one third-order step r(1 + e/3 + 2 e^2/9),
+// e = 1 - h r^3, from a single-precision value.
 __device__ __forceinline__ double rcbrt_r(double h)
 {
     const double r = (double)exp2f(__log2f((float)h) * (-1.f / 3.f));
@@ -358,7 +360,7 @@ template <typename real>
 __device__ __forceinline__ real friction_depth(int law, real fric, real hb, real eps, real hwet)
 {
     if constexpr (sizeof(real) == 8) {
-        if (at_least(hb, hwet)) {   // k = 1/h
+        if (at_least(hb, hwet) && (law != kFricManning || in_single_range(hb))) {   // k = 1/h
             if (law == kFricManning) {
                 const real r = rcbrt_r(hb), r3 = r * r * r;
                 return fric * (r3 * r3 * r);

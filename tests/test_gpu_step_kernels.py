@@ -213,6 +213,25 @@ def test_fp64_elementary_functions(op, lo, hi, ulp):
     assert err.max() <= ulp, (err.max(), x[err.argmax()])
 
 
+@pytest.mark.parametrize("depth,eps", [(1e-39, 1e-160), (1e-20, 1e-90)])
+def test_manning_friction_below_single_precision(depth, eps):
+    """Films thinner than single precision holds, deeper than eps^(1/4): the
+    friction's h^(-7/3) takes the double-precision root, and the state stays
+    finite and follows the oracle."""
+    from paper_1611_05984_gb300 import celeris
+    s = sc.flat_basin(40, 36, 1.0, 1.0, 1e-3, model=1, friction=2, fcoef=0.01, eps=eps)
+    s.z[:, 20:] = 0.0
+    s.w0 = np.where(s.z < 0.0, 0.0, depth)
+    s.w0[:, 24:] = 0.0
+    o = oracle_from(s)
+    g = celeris.from_scenario(s, dtype=torch.float64)
+    o.step(2)
+    g.step(2)
+    assert g.check_finite()
+    for a, b in zip(g.state(), o.state()):
+        np.testing.assert_allclose(a.cpu().numpy(), b, rtol=0, atol=1e-12)
+
+
 def test_fp64_root_at_the_ends():
     from paper_1611_05984_gb300 import celeris
     x = np.array([0.0, -0.0, np.inf, np.nan, -1.0, -np.inf])
