@@ -178,8 +178,9 @@ typedef struct {
 cel_status cel_get_stats(cel_solver *s, cel_stats *out);
 
 /* Checkpoint: state, AB3/AM4 history, step count and time, enough for a
- * bit-exact resume.  Device buffer of cel_checkpoint_bytes.  Asynchronous
- * (save) / synchronises (load reads the header). */
+ * bit-exact resume.  Device buffer of cel_checkpoint_bytes, equal byte for
+ * byte for equal runs (padding and gaps are 0).  Asynchronous (save) /
+ * synchronises (load reads the header). */
 cel_status cel_checkpoint_bytes(const cel_solver *s, size_t *bytes);
 cel_status cel_save_checkpoint(cel_solver *s, void *dst_dev, size_t bytes);
 cel_status cel_load_checkpoint(cel_solver *s, const void *src_dev, size_t bytes);

@@ -896,10 +896,20 @@ cel_status cel_save_checkpoint(cel_solver *s, void *dst_dev, size_t bytes)
     CkptPart parts[32];
     int np = ckpt_parts(s, parts);
     size_t off = align256(sizeof(CkptHeader));
+    CEL_CUDA(s, cudaMemsetAsync(dst + sizeof(h), 0, off - sizeof(h), s->stream), "checkpoint");
     for (int k = 0; k < np; k++) {
         CEL_CUDA(s, cudaMemcpyAsync(dst + off, s->ws + parts[k].off_ws, parts[k].bytes, cudaMemcpyDeviceToDevice,
                                     s->stream), "checkpoint");
-        off += align256(parts[k].bytes);
+        // the rows' padding and the gap to the next part, which hold nothing of the state, as 0
+        const Geo &G = s->geo;
+        const bool col = parts[k].off_ws == s->lay.Qc[s->pcur];
+        const size_t pitch = (size_t)(col ? G.py : G.px) * s->es, used = (size_t)(col ? G.ny : G.nx) * s->es;
+        if (pitch > used)
+            CEL_CUDA(s, cudaMemset2DAsync(dst + off + used, pitch, 0, pitch - used, col ? G.nx : G.ny, s->stream),
+                     "checkpoint");
+        const size_t next = off + align256(parts[k].bytes), end = off + parts[k].bytes;
+        if (next > end) CEL_CUDA(s, cudaMemsetAsync(dst + end, 0, next - end, s->stream), "checkpoint");
+        off = next;
     }
     return CEL_OK;
 }

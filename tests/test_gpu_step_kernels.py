@@ -97,6 +97,29 @@ def test_tile_edges_and_remainders(prec, nx, ny):
     _match(s, prec, 5)
 
 
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("nx,ny,K", [(95, 71, 0), (33, 9, 1), (129, 65, 2)])
+def test_checkpoints_of_identical_runs_are_identical(nx, ny, K, prec):
+    """Odd widths: a checkpoint holds whole padded rows, and its padding is 0
+    whatever the kernels left there (a lane's second cell beyond an odd width)
+    and whatever the buffers held before."""
+    from paper_1611_05984_gb300 import celeris
+
+    def run(scale):
+        s = sc.flat_basin(nx, ny, 1.0, 2.0, 0.01, K=K, friction=1, fcoef=0.01, eps=1e-8)
+        s.w0 = scale * np.add.outer(np.sin(0.3 * np.arange(ny)), np.cos(0.2 * np.arange(nx)))
+        s.P0 = s.Q0 = 0.3 * s.w0
+        g = celeris.from_scenario(s, dtype=torch.float64 if prec == "f64" else torch.float32)
+        g.step(5)
+        return g.checkpoint().cpu().numpy()
+    first = run(0.1)
+    run(0.17)
+    np.testing.assert_array_equal(run(0.1), first)
+    es, px = (8, (nx + 31) // 32 * 32) if prec == "f64" else (4, (nx + 31) // 32 * 32)
+    rows = first[256:256 + ny * px * es].view(np.float64 if prec == "f64" else np.float32).reshape(ny, px)   # w
+    assert not rows[:, nx:].any()
+
+
 @pytest.mark.parametrize("K,model", [(0, 0), (2, 0), (1, 1)])
 def test_carries_correctors_and_shallow_water_across_tiles(K, model):
     """The predictor-only carries, two corrector stages and the shallow-water
