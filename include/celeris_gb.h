@@ -411,7 +411,9 @@ cel_status cel_ensemble_graph_steps(const cel_ensemble *e, int64_t *steps);
  * word and the launch ends at the next barrier, leaving the members' states
  * undefined.  cel_ensemble_check synchronises the ensemble's stream and
  * returns CEL_ERR_TIMEOUT if that happened (the words are cleared).
- * CEL_ERR_CUDA if no block of the launch fits an SM.  Off by default. */
+ * CEL_ERR_CUDA if no block of the launch fits an SM.  Off by default, and
+ * slower in single precision than the default's replayed cycles (64 beaches
+ * 1.46 against 0.97 ms per step; double precision 1 % slower). */
 cel_status cel_ensemble_use_persistent(cel_ensemble *e, int32_t enable, double timeout_ms);
 /* Steps taken by persistent launches since cel_ensemble_create. */
 cel_status cel_ensemble_persistent_steps(const cel_ensemble *e, int64_t *steps);

@@ -464,7 +464,9 @@ class Ensemble:
     def use_persistent(self, enable: bool = True, timeout_ms: float = 1000.0):
         """Take each call's steps in one persistent cooperative launch where
         the captured cycle's conditions hold (cel_ensemble_use_persistent);
-        every grid-wide wait is bounded by timeout_ms."""
+        every grid-wide wait is bounded by timeout_ms.  Slower than the
+        default, the replayed cycles (64 single-precision beaches 1.46 against
+        0.97 ms per step)."""
         st = self.L.cel_ensemble_use_persistent(self._h, int(bool(enable)), float(timeout_ms))
         if st != CEL_OK:
             raise CelerisError(st, self.L.cel_ensemble_last_error(self._h).decode())

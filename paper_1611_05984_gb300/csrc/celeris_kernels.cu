@@ -8,8 +8,9 @@
 //
 // Per step and per stage (predictor, then K corrector iterations) three
 // kernels run:
-//   k_stencil  one tile per thread block (32x32 in FP64; in FP32
-//              k_stencil_pair, celeris_stencil_f32.cuh): stages w, P, Q (+2
+//   k_stencil  one tile per thread block (32x32 in FP64 and in the persistent
+//              ensemble launch; in FP32 otherwise k_stencil_pair,
+//              celeris_stencil_f32.cuh): stages w, P, Q (+2
 //              ghost layers produced in shared memory from the boundary
 //              rules) and the bed corners, computes the face fluxes, then per
 //              cell E, F, G, F*, G*, friction and the time update; writes
@@ -424,9 +425,7 @@ struct StencilSmem {
 // P^{n+1} - P^n from the increment of U*, which equals recomputing U*^n from
 // P^n by Eq. 23 but keeps the rounding relative to the increment.
 template <typename real>
-struct Carry {
-    real a, b, r1, r2, p1, p2, Y;
-};
+using Carry = CarryV<real>;
 
 // The history a stage reads, loaded at the top of a cell's iteration so the
 // loads are in flight while the cell's right side is computed.
@@ -617,8 +616,9 @@ struct SharedOrigin {
 // Fluxes through faces f0 .. f1 - 1 of one row (kX: x-faces, r the row) or
 // one column (y-faces, r the column) of the staged tile.
 template <typename real, int TY, bool kX>
-__device__ __forceinline__ void sweep_faces(StencilSmem<real, TY> &sm, const Coef<real> &C, int r, int f0, int f1)
+__device__ __forceinline__ void sweep_faces(StencilSmem<real, TY> &sm, const StencilArgs<real> &A, int r, int f0, int f1)
 {
+    const Coef<real> &C = A.c;
     // strides along the sweep, and from a face's first corner to its second
     constexpr int sq = kX ? 1 : kStride, sc = kX ? 1 : kCornerStride, sc2 = kX ? kCornerStride : 1;
     constexpr int sf = kX ? 1 : kTile, sv = kX ? TY * (kTile + 1) : (TY + 1) * kTile;
@@ -644,7 +644,8 @@ __device__ __forceinline__ void sweep_faces(StencilSmem<real, TY> &sm, const Coe
         const real q[3] = {pw[2 * sq], pn[2 * sq], pt[2 * sq]};
         sweep.next(C.th2, q, Bf, Bn, lo, hn, dlo, dn);
         real H[3];
-        face_flux_step(C.g, C.eps, C.hwet, hi[0], hi[1], hi[2], dhi, lo[0], lo[1], lo[2], dlo, H);
+        if constexpr (sizeof(real) == 4) flux_v<real>(A, hi, dhi, lo, dlo, H);
+        else face_flux_step(C.g, C.eps, C.hwet, hi[0], hi[1], hi[2], dhi, lo[0], lo[1], lo[2], dlo, H);
         out[0] = H[0];
         out[kX ? sv : 2 * sv] = H[1];   // momentum normal to the face
         out[kX ? 2 * sv : sv] = H[2];
@@ -762,17 +763,17 @@ __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const O
     if constexpr (TY == kTile) {
         const int lane = tid & 31, wq = (tid >> 5) & 3;
         const int f0 = wq * 8, f1 = wq == 3 ? kTile + 1 : f0 + 8;
-        if (tid < 4 * 32) sweep_faces<real, TY, true>(sm, C, lane, f0, f1);
-        else sweep_faces<real, TY, false>(sm, C, lane, f0, f1);
+        if (tid < 4 * 32) sweep_faces<real, TY, true>(sm, A, lane, f0, f1);
+        else sweep_faces<real, TY, false>(sm, A, lane, f0, f1);
     } else {
         constexpr int nxf = TY * (kTile + 1), nx32 = (nxf + 31) / 32 * 32, nyf = (TY + 1) * kTile;
         for (int k = tid; k < nx32 + nyf; k += kStencilThreads) {
             if (k < nxf) {
                 const int r = k / (kTile + 1), f = k - r * (kTile + 1);
-                sweep_faces<real, TY, true>(sm, C, r, f, f + 1);
+                sweep_faces<real, TY, true>(sm, A, r, f, f + 1);
             } else if (k >= nx32) {
                 const int f = (k - nx32) / kTile, c = (k - nx32) % kTile;
-                sweep_faces<real, TY, false>(sm, C, c, f, f + 1);
+                sweep_faces<real, TY, false>(sm, A, c, f, f + 1);
             }
         }
     }
@@ -815,9 +816,17 @@ __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const O
         const real E = div(0);
         // bed slope: the face beds' difference is half that of the corner sums
         const real sx = sub_r(add_r(c10, c11), add_r(c00, c01)), sy = sub_r(add_r(c01, c11), add_r(c00, c10));
-        real F = fma(mul_r(hb, -C.hgx), sx, div(1));
-        real Gq = fma(mul_r(hb, -C.hgy), sy, div(2));
-        if (friction != kFricNone) {   // Eq. 31-32 with the Eq. 14 device
+        real F, Gq;
+        if constexpr (sizeof(real) == 4) {   // the two-cell tiles' order, and their bits
+            const real gh = mul2(kc<real>(A, kcMHalfG), hb);
+            F = fma2(mul2(gh, sx), rdx, div(1));
+            Gq = fma2(mul2(gh, sy), rdy, div(2));
+            if (friction != kFricNone) friction_v<real>(A, friction, hb, P0, Q0, F, Gq);
+        } else {
+            F = fma(mul_r(hb, -C.hgx), sx, div(1));
+            Gq = fma(mul_r(hb, -C.hgy), sy, div(2));
+        }
+        if (sizeof(real) == 8 && friction != kFricNone) {   // Eq. 31-32 with the Eq. 14 device
             const real fm = mul_r(friction_depth(friction, C.fric, hb, eps, C.hwet),
                                   sqrt_r(fma(P0, P0, mul_r(Q0, Q0))));
             F = fma(-fm, P0, F);
@@ -826,7 +835,20 @@ __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const O
         real Fs = real(0), Gs = real(0);
         const int od = (cy + 1) * kDStride + cx + 1;
         const real dd = sm.d[od];
-        if (bsnq) {
+        if (sizeof(real) == 4 && bsnq) {
+            if constexpr (sizeof(real) == 4) {
+                constexpr int S1 = kStride;
+                const real ddx = mul2(sub2(sm.d[od + 1], sm.d[od - 1]), kc<real>(A, kcHrdx));
+                const real ddy = mul2(sub2(sm.d[od + kDStride], sm.d[od - kDStride]), kc<real>(A, kcHrdy));
+                auto around = [&](const real *p) {
+                    return Around<real>{p[0], p[1], p[-1], p[S1], p[-S1], p[S1 + 1], p[S1 - 1], p[1 - S1], p[-1 - S1],
+                                        p[2], p[-2], p[2 * S1], p[-2 * S1]};
+                };
+                eta_terms_v(A, around(sm.w + o), dd, ddx, ddy, F, Gq);
+                Fs = mixed_term_v(A, around(sm.Q + o), dd, ddx, ddy);
+                Gs = mixed_term_v(A, around(sm.P + o), dd, ddx, ddy);
+            }
+        } else if (bsnq) {
             const real dDx = sub_r(sm.d[od + 1], sm.d[od - 1]), dDy = sub_r(sm.d[od + kDStride], sm.d[od - kDStride]);
             const real d2 = mul_r(dd, dd);
             const real *W = sm.w + o;
@@ -858,10 +880,17 @@ __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const O
         }
         real w1 = w0, dU = real(0), dV = real(0);
         if (valid) {
-            real dw = advance<real, kSpec>(A, 0, w0, E, real(0), kr, cw);
-            w1 = stage_kind<kSpec>(A) == kAM4 ? dw : add_r(w0, dw);   // the AM4 base of w holds w^n
-            dU = advance<real, kSpec>(A, 1, real(0), F, Fs, kr, cu);
-            dV = advance<real, kSpec>(A, 2, real(0), Gq, Gs, kr, cv);
+            if constexpr (sizeof(real) == 4) {
+                const real dw = advance_v<real, kSpec>(A, 0, w0, E, 0.f, (unsigned)kr, cw, true);
+                w1 = kSpec != 0 ? dw : add2(w0, dw);
+                dU = advance_v<real, kSpec>(A, 1, 0.f, F, Fs, (unsigned)kr, cu, true);
+                dV = advance_v<real, kSpec>(A, 2, 0.f, Gq, Gs, (unsigned)kr, cv, true);
+            } else {
+                real dw = advance<real, kSpec>(A, 0, w0, E, real(0), kr, cw);
+                w1 = stage_kind<kSpec>(A) == kAM4 ? dw : add_r(w0, dw);   // the AM4 base of w holds w^n
+                dU = advance<real, kSpec>(A, 1, real(0), F, Fs, kr, cu);
+                dV = advance<real, kSpec>(A, 2, real(0), Gq, Gs, kr, cv);
+            }
             if (w1 < Bb) w1 = Bb;   // Reading A-D1
             if (sponge_tile) {
                 real gam = sponge_gamma<real>(C, G, i, j);
@@ -906,26 +935,13 @@ __global__ void __launch_bounds__(kStencilThreads, 2) k_stencil(const __grid_con
 }
 
 // FP32 (celeris_stencil_f32.cuh): 64 columns and 4 kR rows per block.
-struct BlockBarrier {
-    __device__ __forceinline__ void operator()() const { __syncthreads(); }
-};
-// The barrier of one half of a 256-thread block.
-struct HalfBarrier {
-    int id;
-    __device__ __forceinline__ void operator()() const
-    {
-        asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kPThreads) : "memory");
-    }
-};
-
 template <int kSpec, int kR>
 __global__ void __launch_bounds__(kPThreads, 4) k_stencil_pair(const __grid_constant__ StencilArgs<float> A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     dependent_launch_wait();
     if (releases_early()) dependent_launch_release();
-    stencil_tile_pair<kSpec, kR>(A, blockIdx.x * kPW, blockIdx.y * PairSmem<kR>::TH, smem_raw, threadIdx.x,
-                                 BlockBarrier());
+    stencil_tile_pair<kSpec, kR>(A, blockIdx.x * kPW, blockIdx.y * PairSmem<kR>::TH, smem_raw);
     if (!releases_early()) dependent_launch_release();
 }
 
@@ -968,8 +984,7 @@ __global__ void __launch_bounds__(kPThreads, 4)
     const int2 d = desc[blockIdx.x];
     load_args(A, args + d.x);
     __syncthreads();
-    stencil_tile_pair<kSpec, kPairRows>(A, (d.y & 0xffff) * kPW, (d.y >> 16) * PairSmem<kPairRows>::TH, smem_raw,
-                                        threadIdx.x, BlockBarrier());
+    stencil_tile_pair<kSpec, kPairRows>(A, (d.y & 0xffff) * kPW, (d.y >> 16) * PairSmem<kPairRows>::TH, smem_raw);
 }
 
 // ------------------------------------------------------------ line solves
@@ -1854,36 +1869,16 @@ __device__ __noinline__ bool grid_sync(unsigned *bar, unsigned expect, long long
 // The arguments sit in shared memory and nothing the work stores aliases
 // them, which the compiler is told so that it keeps them in registers
 // across the global stores.
-template <int kSpec>
-__device__ __noinline__ void persist_tile(const StencilArgs<double> &__restrict__ A, const int *origin,
+template <typename real, int kSpec>
+__device__ __noinline__ void persist_tile(const StencilArgs<real> &__restrict__ A, const int *origin,
                                           unsigned char *smem_raw)
 {
     __builtin_assume(__isShared(&A));
-    stencil_tile<double, kSpec, kTile>(A, SharedOrigin{origin}, smem_raw);
+    stencil_tile<real, kSpec, kTile>(A, SharedOrigin{origin}, smem_raw);
 }
 
-// A tile's arguments and origin, behind the tiles' shared memory.
-template <typename real>
-struct __align__(16) PersistTile {
-    StencilArgs<real> A;
-    int origin[2];
-};
-
-// FP32: each half of the block takes a tile of its own (kPThreads threads).
 // The launch's shared memory is named here, not passed: through pointers the
 // accesses would be generic ones.
-constexpr int kPersistHalves = kStencilThreads / kPThreads;
-template <int kSpec>
-__device__ __noinline__ void persist_tile_pair()
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int half = threadIdx.x / kPThreads;
-    const PersistTile<float> &t =
-        reinterpret_cast<const PersistTile<float> *>(smem_raw + kPersistHalves * sizeof(PairSmem<kPairRows>))[half];
-    stencil_tile_pair<kSpec, kPairRows>(t.A, t.origin[0], t.origin[1], smem_raw + half * sizeof(PairSmem<kPairRows>),
-                                        threadIdx.x & (kPThreads - 1), HalfBarrier{1 + half});
-}
-
 template <typename real, int M>
 __device__ __noinline__ void persist_line(int slot, int line, int tid, int wbase, bool valid)
 {
@@ -1894,6 +1889,18 @@ __device__ __noinline__ void persist_line(int slot, int line, int tid, int wbase
     line_solve_reg<real, M, 0>(Al[slot], line, L, tid, wbase, valid);
 }
 
+// A tile's arguments and origin, behind the tile's shared memory.
+template <typename real>
+struct __align__(16) PersistTile {
+    StencilArgs<real> A;
+    int origin[2];
+};
+template <typename real>
+__host__ __device__ constexpr size_t persist_smem()
+{
+    return (sizeof(StencilSmem<real, kTile>) + 15) / 16 * 16 + sizeof(PersistTile<real>);
+}
+
 // A descriptor or entry index out of range: recorded once in bar[3] (code
 // in the top byte, the index below), and the work it names is skipped.
 __device__ __forceinline__ void persist_flag(unsigned *bar, unsigned code, unsigned info)
@@ -1901,66 +1908,54 @@ __device__ __forceinline__ void persist_flag(unsigned *bar, unsigned code, unsig
     atomicCAS(bar + 3, 0u, (code << 24) | (info & 0xffffffu));
 }
 
+// FP32 takes a cell per thread here (32 x 32 tiles, 64 registers) with the
+// arithmetic of the two-cell tiles and the same bits: the line phases live on
+// warps, and two blocks per SM of the two-cell tiles' 128 registers have half
+// as many as four of these (64 beaches 1.46 ms per step against 1.72, 256
+// beaches 5.36 against 6.32).  The captured batched launches, the default,
+// take 0.97 and 3.50.
+//
 // One launch for nsteps lockstep steps of an ensemble: the work of each
 // batched launch (ghost tables; per stage the stencil tiles, then the line
 // solves) spread over the resident blocks, a grid-wide barrier where a
 // batched launch would end.  Every block runs the same loop, so each takes
 // every barrier.
 template <typename real>
-__host__ __device__ constexpr size_t persist_smem()
-{
-    return sizeof(real) == 4 ? kPersistHalves * (sizeof(PairSmem<kPairRows>) + sizeof(PersistTile<real>))
-                             : (sizeof(StencilSmem<double, kTile>) + 15) / 16 * 16 + sizeof(PersistTile<real>);
-}
-
-template <typename real>
-__global__ void __launch_bounds__(kStencilThreads, 2)
+__global__ void __launch_bounds__(kStencilThreads, sizeof(real) == 4 ? 4 : 2)
     k_ensemble_persistent(const __grid_constant__ PersistArgs<real> P)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    // tiles side by side in the block, and threads of each
-    constexpr int kSide = sizeof(real) == 4 ? kPersistHalves : 1, kOwn = kStencilThreads / kSide;
-    constexpr int kTX = sizeof(real) == 4 ? kPW : kTile, kTY = sizeof(real) == 4 ? PairSmem<kPairRows>::TH : kTile;
-    static_assert(sizeof(PairSmem<kPairRows>) % 16 == 0, "tiles side by side keep their alignment");
-    PersistTile<real> *tile =
-        reinterpret_cast<PersistTile<real> *>(smem_raw + persist_smem<real>() - kSide * sizeof(PersistTile<real>));
-    __shared__ int item[kSide];
+    PersistTile<real> &tile = *reinterpret_cast<PersistTile<real> *>(smem_raw + persist_smem<real>() - sizeof(PersistTile<real>));
+    StencilArgs<real> &As = tile.A;
+    int *origin = tile.origin;
+    __shared__ int item;
     // the line phases reuse the stencil's shared memory: a slot's arguments,
     // then the values that cross warps
-    static_assert(sizeof(LineArgs<real>) * (kStencilThreads / 32) + sizeof(LineShared<real>) <= persist_smem<real>(),
+    static_assert(sizeof(LineArgs<real>) * (kStencilThreads / 32) + sizeof(LineShared<real>) <=
+                      sizeof(StencilSmem<real, kTile>),
                   "line phase shared memory");
     LineArgs<real> *Al = reinterpret_cast<LineArgs<real> *>(smem_raw);
     if (P.barrier_only) {
         grid_sync(P.bar, P.expect, P.timeout_ns);
         return;
     }
-    // Tiles and line passes go to whoever is free (a counter per phase, three
-    // used in turn), as the hardware hands out the blocks of a launch, so that
-    // a phase ends when its work does and not with its slowest block's fixed
-    // share.  Tiles side by side in a block are taken one by one, each by its
-    // own threads; line passes kLineChunk at a time, whose descriptors and
-    // arguments are fetched together: with two blocks on an SM a pass's chain
-    // of counter, descriptor, arguments and operands is little hidden.
-    // 64 beaches, FP32: 1.80 -> 1.66 ms per step with this and the shared
-    // memory named in the calls (the captured batched launches: 0.99).
+    // Tiles and line passes go to blocks as they free up (a counter per
+    // phase, three used in turn), as the hardware hands out the blocks of a
+    // launch, so that a phase ends when its work does and not with its
+    // slowest block's fixed share.
+    constexpr int kParts = sizeof(real) == 4 ? kPairCols / kTile : 1;   // 32 x 32 tiles of one descriptor's
+    // Line passes are taken kLineChunk at a time, whose descriptors and
+    // arguments are fetched together, to hide some of a pass's chain of counter,
+    // descriptor, arguments and operands (FP32, ms per step with 1 / 2 / 4 / 8 at
+    // a time: 64 beaches 1.53 / 1.46 / 1.47 / 1.53, 256 beaches 5.68 / 5.39 / 5.37
+    // / 5.39; FP64 no difference).
     constexpr int kLineChunk = 4;
     int phase = 0;
-    const int half = threadIdx.x / kOwn, own_tid = threadIdx.x - half * kOwn;
-    auto half_sync = [&]() {
-        if constexpr (kSide > 1) HalfBarrier{1 + half}();
-        else __syncthreads();
-    };
-    auto next_tile = [&]() -> int {
-        half_sync();   // the tile's threads are done with the one before
-        if (own_tid == 0) item[half] = atomicAdd(P.work + phase % 3, 1);
-        half_sync();
-        return item[half];
-    };
-    auto next_chunk = [&]() -> int {
+    auto next_item = [&]() -> int {
+        __syncthreads();   // the block is done with its previous item
+        if (threadIdx.x == 0) item = atomicAdd(P.work + phase % 3, 1);
         __syncthreads();
-        if (threadIdx.x == 0) item[0] = atomicAdd(P.work + phase % 3, 1);
-        __syncthreads();
-        return item[0] * kLineChunk;
+        return item;
     };
     auto end_phase = [&]() -> bool {
         const bool ok = grid_sync(P.bar, P.expect, P.timeout_ns, P.work + (phase + 2) % 3);
@@ -1986,36 +1981,30 @@ __global__ void __launch_bounds__(kStencilThreads, 2)
             const unsigned char *ent = P.entries + (size_t)ei * P.entry_bytes;
             const StencilArgs<real> *sa = reinterpret_cast<const StencilArgs<real> *>(ent);
             const int spec = P.spec[stage];
-            for (int t = next_tile(); t < P.tiles; t = next_tile()) {
-                const int own = own_tid;
-                const int2 d = P.tile_desc[t];
-                bool ok = d.x >= 0 && d.x < P.nmembers;
-                if (!ok && own == 0) persist_flag(P.bar, 1u, (unsigned)t);
-                if (ok) {
-                    if (own == 0) {
-                        tile[half].origin[0] = (d.y & 0xffff) * kTX;
-                        tile[half].origin[1] = (d.y >> 16) * kTY;
-                    }
-                    const int nw = (int)(sizeof(StencilArgs<real>) / sizeof(int));
-                    int *dst = reinterpret_cast<int *>(&tile[half].A);
-                    const int *src = reinterpret_cast<const int *>(sa + d.x);
-                    for (int k = own; k < nw; k += kOwn) dst[k] = src[k];
+            for (int t = next_item(); t < kParts * P.tiles; t = next_item()) {
+                const int2 d = P.tile_desc[t / kParts];
+                const int x0 = (d.y & 0xffff) * kParts * kTile, y0 = (d.y >> 16) * kTile;
+                if (d.x < 0 || d.x >= P.nmembers) {
+                    if (threadIdx.x == 0) persist_flag(P.bar, 1u, (unsigned)(t / kParts));
+                    continue;
                 }
-                half_sync();
-                if (ok && ((d.y & 0xffff) * kTX >= tile[half].A.geo.nx || (d.y >> 16) * kTY >= tile[half].A.geo.ny)) {
-                    if (own == 0) persist_flag(P.bar, 2u, (unsigned)t);
-                    ok = false;
+                if (threadIdx.x == 0) {
+                    origin[0] = x0 + t % kParts * kTile;
+                    origin[1] = y0;
                 }
-                if (!ok) continue;   // this tile's threads wait at the next item
-                if constexpr (sizeof(real) == 4) {
-                    if (spec == 1) persist_tile_pair<1>();
-                    else if (spec == 2) persist_tile_pair<2>();
-                    else persist_tile_pair<0>();
-                } else {
-                    if (spec == 1) persist_tile<1>(tile[half].A, tile[half].origin, smem_raw);
-                    else if (spec == 2) persist_tile<2>(tile[half].A, tile[half].origin, smem_raw);
-                    else persist_tile<0>(tile[half].A, tile[half].origin, smem_raw);
+                load_args(As, sa + d.x);
+                __syncthreads();
+                if (x0 >= As.geo.nx || y0 >= As.geo.ny) {
+                    if (threadIdx.x == 0) persist_flag(P.bar, 2u, (unsigned)(t / kParts));
+                    continue;
                 }
+                if (x0 + t % kParts * kTile >= As.geo.nx) continue;   // the tile's half beyond the grid
+                if (spec == 1)
+                    persist_tile<real, 1>(As, origin, smem_raw);
+                else if (spec == 2)
+                    persist_tile<real, 2>(As, origin, smem_raw);
+                else
+                    persist_tile<real, 0>(As, origin, smem_raw);
             }
             if (!end_phase()) return;
             const LineArgs<real> *la = reinterpret_cast<const LineArgs<real> *>(ent + P.sarg_bytes);
@@ -2025,60 +2014,58 @@ __global__ void __launch_bounds__(kStencilThreads, 2)
                 while (P.run_pass0[r + 1] <= p) r++;
                 return r;
             };
-            for (int c = next_chunk(); c < passes; c = next_chunk()) {
-                if (threadIdx.x < 8 * kLineChunk && c + (threadIdx.x >> 3) < passes) {
-                  const int p = c + (threadIdx.x >> 3), r = run_of(p), G = kStencilThreads / P.run_threads[r];
-                  const int k = (p - P.run_pass0[r]) * G + (threadIdx.x & 7);
-                  if ((threadIdx.x & 7) < G && k < P.run_lines[r]) {
-                      const int2 d = P.run_desc[r][k];
-                      if (d.x >= 0 && d.x < P.run_nfam[r]) {
-                          const char *src = reinterpret_cast<const char *>(la + P.run_first[r] + d.x);
-                          for (int b = 0; b < (int)sizeof(LineArgs<real>) + 127; b += 128)
-                              asm volatile("prefetch.global.L1 [%0];" ::"l"(src + min(b, (int)sizeof(LineArgs<real>) - 4)));
-                      }
-                  }
+            for (int c = kLineChunk * next_item(); c < passes; c = kLineChunk * next_item()) {
+                if (kLineChunk > 1 && threadIdx.x < 8 * kLineChunk && c + (threadIdx.x >> 3) < passes) {
+                    const int p = c + (threadIdx.x >> 3), r = run_of(p), G = kStencilThreads / P.run_threads[r];
+                    const int k = (p - P.run_pass0[r]) * G + (threadIdx.x & 7);
+                    if ((threadIdx.x & 7) < G && k < P.run_lines[r]) {
+                        const int2 d = P.run_desc[r][k];
+                        if (d.x >= 0 && d.x < P.run_nfam[r]) {
+                            const char *src = reinterpret_cast<const char *>(la + P.run_first[r] + d.x);
+                            for (int b = 0; b < (int)sizeof(LineArgs<real>) + 127; b += 128)
+                                asm volatile("prefetch.global.L1 [%0];" ::"l"(src + min(b, (int)sizeof(LineArgs<real>) - 4)));
+                        }
+                    }
                 }
                 for (int p = c; p < min(c + kLineChunk, passes); p++) {
                     if (p > c) __syncthreads();   // the block is done with the pass before
                     const int r = run_of(p), q = p - P.run_pass0[r];
-                    {
-                        // G lines of T threads side by side; threads past G T only pass the barriers
-                        const int T = P.run_threads[r], G = kStencilThreads / T, nl = P.run_lines[r];
-                        const int slot = threadIdx.x / T, tid = threadIdx.x - slot * T;
-                        const int line_q = q * G + slot;
-                        const bool valid = slot < G && line_q < nl;
-                        const int own = valid ? slot : 0;   // a spare slot takes slot 0's arguments
-                        bool bad = false;
-                        if (slot < G) {
-                            const int2 d = P.run_desc[r][valid ? line_q : q * G];
-                            bad = d.x < 0 || d.x >= P.run_nfam[r];
-                            if (bad && tid == 0) persist_flag(P.bar, 4u, (unsigned)(r * 65536 + q));
-                            if ((valid || slot == 0) && !bad) {
-                                const int nw = (int)(sizeof(LineArgs<real>) / sizeof(int));
-                                int *dst = reinterpret_cast<int *>(&Al[slot]);
-                                const int *src = reinterpret_cast<const int *>(la + P.run_first[r] + d.x);
-                                for (int k = tid; k < nw; k += T) dst[k] = src[k];
-                            }
-                        }
-                        if (__syncthreads_or(bad)) continue;   // skip the pass (the block's decision)
-                        // the run's segment length picks the instance, the same
-                        // for every slot, and the run's lines are all of one
-                        // model: the solve's barriers are the block's, and the
-                        // shallow-water model takes none
+                    // G lines of T threads side by side; threads past G T only pass the barriers
+                    const int T = P.run_threads[r], G = kStencilThreads / T, nl = P.run_lines[r];
+                    const int slot = threadIdx.x / T, tid = threadIdx.x - slot * T;
+                    const int line_q = q * G + slot;
+                    const bool valid = slot < G && line_q < nl;
+                    const int own = valid ? slot : 0;   // a spare slot takes slot 0's arguments
+                    bool bad = false;
+                    if (slot < G) {
                         const int2 d = P.run_desc[r][valid ? line_q : q * G];
-                        const bool bad2 = slot < G && (d.y < 0 || d.y >= Al[own].nlines || Al[own].nseg > T ||
-                                                       (Al[own].nseg & 31) != 0 || Al[own].mshift != P.run_mshift[r] ||
-                                                       Al[own].identity != P.run_identity[r]);
-                        if (bad2 && tid == 0) persist_flag(P.bar, 5u, (unsigned)(r * 65536 + q));
-                        if (__syncthreads_or(bad2)) continue;
-                        const int wb = slot * (T >> 5);
-                        if (P.run_mshift[r] == 3)
-                            persist_line<real, 8>(own, d.y, tid, wb, valid);
-                        else if (P.run_mshift[r] == 2)
-                            persist_line<real, 4>(own, d.y, tid, wb, valid);
-                        else
-                            persist_line<real, 2>(own, d.y, tid, wb, valid);
+                        bad = d.x < 0 || d.x >= P.run_nfam[r];
+                        if (bad && tid == 0) persist_flag(P.bar, 4u, (unsigned)(r * 65536 + q));
+                        if ((valid || slot == 0) && !bad) {
+                            const int nw = (int)(sizeof(LineArgs<real>) / sizeof(int));
+                            int *dst = reinterpret_cast<int *>(&Al[slot]);
+                            const int *src = reinterpret_cast<const int *>(la + P.run_first[r] + d.x);
+                            for (int k = tid; k < nw; k += T) dst[k] = src[k];
+                        }
                     }
+                    if (__syncthreads_or(bad)) continue;   // skip the pass (the block's decision)
+                    // the run's segment length picks the instance, the same
+                    // for every slot, and the run's lines are all of one
+                    // model: the solve's barriers are the block's, and the
+                    // shallow-water model takes none
+                    const int2 d = P.run_desc[r][valid ? line_q : q * G];
+                    const bool bad2 = slot < G && (d.y < 0 || d.y >= Al[own].nlines || Al[own].nseg > T ||
+                                                   (Al[own].nseg & 31) != 0 || Al[own].mshift != P.run_mshift[r] ||
+                                                   Al[own].identity != P.run_identity[r]);
+                    if (bad2 && tid == 0) persist_flag(P.bar, 5u, (unsigned)(r * 65536 + q));
+                    if (__syncthreads_or(bad2)) continue;
+                    const int wb = slot * (T >> 5);
+                    if (P.run_mshift[r] == 3)
+                        persist_line<real, 8>(own, d.y, tid, wb, valid);
+                    else if (P.run_mshift[r] == 2)
+                        persist_line<real, 4>(own, d.y, tid, wb, valid);
+                    else
+                        persist_line<real, 2>(own, d.y, tid, wb, valid);
                 }
             }
             if (!end_phase()) return;

@@ -533,12 +533,12 @@ __device__ __forceinline__ void prefetch_history(const StencilArgs<float> &A, in
     }
 }
 
-// One tile, kPThreads threads (tid 0 .. kPThreads - 1), bar() the barrier of
-// these threads.
-template <int kSpec, int kR, typename Bar>
+// One tile, by a block of kPThreads threads.
+template <int kSpec, int kR>
 __device__ __forceinline__ void stencil_tile_pair(const StencilArgs<float> &A, const int x0, const int y0,
-                                                  unsigned char *smem_raw, const int tid, const Bar &bar)
+                                                  unsigned char *smem_raw)
 {
+    const int tid = threadIdx.x;
     const StencilArgs<float> &A0 = A;
     using S = PairSmem<kR>;
     constexpr int TH = S::TH;
@@ -618,7 +618,7 @@ __device__ __forceinline__ void stencil_tile_pair(const StencilArgs<float> &A, c
         }
         cp_async_wait_all();
     }
-    bar();
+    __syncthreads();
 
     // ---- 2. ghost layers (Sec. 2.4): x-sides over interior rows, then
     //         y-sides over every column, so corners come by composition.
@@ -645,7 +645,7 @@ __device__ __forceinline__ void stencil_tile_pair(const StencilArgs<float> &A, c
         }
     }
     if (southT || northT) {
-        bar();   // the corner columns' x-ghosts
+        __syncthreads();   // the corner columns' x-ghosts
         for (int k = tid; k < 4 * (kPW + 2); k += kPThreads) {
             const int c = 3 + k % (kPW + 2), which = k / (kPW + 2);
             const int gx = x0 - 4 + c, side = which < 2 ? 2 : 3, kk = which & 1;
@@ -666,7 +666,7 @@ __device__ __forceinline__ void stencil_tile_pair(const StencilArgs<float> &A, c
             }
         }
     }
-    if (westT || eastT || southT || northT) bar();
+    if (westT || eastT || southT || northT) __syncthreads();
 
     // ---- 3. the faces at the tile's west and east edges and the depths of
     //         the cells beyond them, for this warp's rows
@@ -948,7 +948,7 @@ __device__ __forceinline__ void stencil_tile_pair(const StencilArgs<float> &A, c
             }
         }
     }
-    bar();
+    __syncthreads();
     if (tid < kPW && x0 + tid < nx) {
         const size_t word = (size_t)(x0 + tid) * G.nwy + (y0 >> 5);
         if constexpr (TH == 32) A.mask_c[word] = sm.col[tid];
