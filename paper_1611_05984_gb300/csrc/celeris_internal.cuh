@@ -32,7 +32,7 @@ constexpr int kDcell = kTile + 2;            // 34 cells of d per tile edge
 constexpr int kDStride = kDcell + 1;
 constexpr int kStencilThreads = 256;
 constexpr int kPairCols = 64, kPairWarps = 4;   // FP32 stencil tile: columns (two per lane), warps
-constexpr int kPairRows = 8;                    // its rows per warp where there are tiles enough
+constexpr int kPairRows = 8;                    // its rows per warp in the ensembles' batched launches
 // An ensemble's stencil tiles, per precision.
 inline int tile_cols(int real_bytes) { return real_bytes == 4 ? kPairCols : kTile; }
 inline int tile_rows(int real_bytes) { return real_bytes == 4 ? kPairRows * kPairWarps : kTile; }
@@ -340,9 +340,12 @@ int dependent_launch();
 // up with two on some SMs and none on others (FP64 gradient of 200 x 150
 // cells, with its Jacobian kernel held to one block per SM as well: 14.4 ms a
 // pass with the release at the start, 10.0 at the end; 601 x 601 FP32 island
-// 838 -> 792 us, 2048 x 2048 beach 4181 -> 4132 us).  Only a grid that leaves
-// most SMs free lets the next kernel start at once (559 x 4 beach 722 us, 733
-// with the release at the end).
+// 838 -> 792 us, 2048 x 2048 beach 4181 -> 4132 us).  Only a stencil grid of at
+// most 64 blocks, which leaves most SMs free, lets the next kernel start at
+// once.  Step in us with the release at the start / at the end, by blocks: FP32
+// 9 (559 x 4) 19.5 / 21.6, 16 18.3 / 18.6, 40 18.8 / 19.1, 64 18.6 / 19.7, 80 19.3
+// / 19.4, 128 23.5 / 20.4, 200 20.9 / 21.7; FP64 8 (64 x 8) 39.6 / 42.4, 32 41.6 /
+// 46.2, 60 47.6 / 53.4, 64 47.5 / 52.8, 128 51.9 / 53.1 and 64.4 / 64.8.
 __device__ __forceinline__ void dependent_launch_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dependent_launch_release()
 {

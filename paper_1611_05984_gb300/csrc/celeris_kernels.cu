@@ -2277,15 +2277,13 @@ template <>
 cudaError_t launch_stencil<float>(const StencilArgs<float> &a, cudaStream_t st)
 {
     // Rows per warp, by the number of 64 x 32 tiles (608 blocks fit the GPU at
-    // once): 8 need the fewest instructions per cell, and win once there are
-    // enough tiles to keep the SMs evenly loaded; fewer rows give more and
-    // shorter blocks.  Step in us with 8 / 4 / 2 rows: 2048 x 2048 (2048
-    // tiles) 272 / - / 277; 1024 x 1024 (512) 89 / 84 / 86; 601 x 601 (190)
-    // 55 / 46 / 46; 512 x 512 (128) 47 / 37 / 37; 256 x 256 (32) 46 / 32 / 26.
+    // once): more rows need fewer instructions per cell, fewer rows give more
+    // and shorter blocks and load the SMs more evenly.  Step in us with 8 / 4 /
+    // 2 rows: 8192 x 8192 (32768 tiles) 3970 / 3889 / -; 2048 x 2048 (2048)
+    // 274 / 260 / 283; 1024 x 1024 (512) 94 / 86 / 90; 601 x 601 (190) 56 / 43 /
+    // 45; 512 x 512 (128) 49 / 37 / 34; 256 x 256 (32) 45 / 31 / 26.
     const long tiles = (long)((a.geo.nx + kPW - 1) / kPW) * ((a.geo.ny + 31) / 32);
-    if (tiles >= 1024) return launch_stencil_pair<kPairRows>(a, st);
-    if (tiles >= 152) return launch_stencil_pair<4>(a, st);
-    return launch_stencil_pair<2>(a, st);
+    return tiles >= 152 ? launch_stencil_pair<4>(a, st) : launch_stencil_pair<2>(a, st);
 }
 
 // The ensemble's batched launches are plain launches: replayed as captured

@@ -75,7 +75,7 @@ def test_a_non_finite_cell_reaches_its_neighbours(field, value, prec):
     assert np.isfinite(w).all()
 
 
-# The FP32 stencil's tiles are 64 columns by 32, 16 or 8 rows (by the number of
+# The FP32 stencil's tiles are 64 columns by 16 or 8 rows (by the number of
 # tiles), the FP64 stencil's 32 columns by 32, 4 or 2 rows: one column or row
 # short of, at and past their edges, odd widths (a lane's second cell outside),
 # and each height.
