@@ -345,7 +345,8 @@ int dependent_launch();
 // once.  Step in us with the release at the start / at the end, by blocks: FP32
 // 9 (559 x 4) 19.5 / 21.6, 16 18.3 / 18.6, 40 18.8 / 19.1, 64 18.6 / 19.7, 80 19.3
 // / 19.4, 128 23.5 / 20.4, 200 20.9 / 21.7; FP64 8 (64 x 8) 39.6 / 42.4, 32 41.6 /
-// 46.2, 60 47.6 / 53.4, 64 47.5 / 52.8, 128 51.9 / 53.1 and 64.4 / 64.8.
+// 46.2, 60 47.6 / 53.4, 64 47.5 / 52.8, 128 51.9 / 53.1 and 64.4 / 64.8 (above
+// 64 blocks either may be the faster).
 __device__ __forceinline__ void dependent_launch_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dependent_launch_release()
 {

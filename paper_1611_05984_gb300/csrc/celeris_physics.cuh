@@ -99,8 +99,8 @@ __device__ __forceinline__ void cu_flux(real g, real eps, real wL, real nL, real
 // on the bit patterns with integer instructions, and reciprocals and roots are
 // refined from the hardware's approximations (Householder's third-order step;
 // Goldschmidt's iteration and a remainder).  2048 x 2048 beach, both stages and the line solves
-// of 2 Euler and 2 full steps: 27.4 ms before, 20.0 ms with these forms (the
-// stencil's FP64 instructions per cell from about 580 to 350).
+// of 2 Euler and 2 full steps: 27.4 ms before, 20.0 ms with these forms, 19.4
+// now (the predictor's DFMA, DADD and DMUL per cell from 425 to 309).
 
 // Single operations, each rounded: where an expression could be contracted
 // into a fused multiply-add in more than one way, the choice is written out

@@ -1,8 +1,8 @@
 // The FP32 stencil stage over one tile: 64 columns, a lane owning two
 // neighbouring cells of a row, a warp kR consecutive rows.
 //
-// The FP32 stencil is bound by instruction issue, so the layout is the one
-// with the fewest instructions per cell:
+// With a cell per thread the FP32 stencil was bound by instruction issue, so
+// the layout is the one with the fewest instructions per cell:
 //   * two cells per lane: additions, multiplications and fused
 //     multiply-adds on both at once (.f32x2), 64-bit loads and stores of
 //     shared and global memory, and one set of addresses, branches and loop
@@ -18,12 +18,13 @@
 // row's one branch, on a negative depth, skips a fix that would change
 // nothing), so tiles of different heights give the same bits.
 //
-// Per cell about 455 thread instructions in the predictor and 410 in the
-// corrector (865 and 800 with a cell per thread and the fluxes in shared
-// memory).  128 registers, no spills, 4 blocks of 128 threads per SM: at 16
-// warps per SM it is bound by the latency of its own chains (0.6 of the issue
-// slots; 0.35 of the FMA pipe).  Mean of both stages, with events around the
-// launches: 2048 x 2048 cells 115 -> 96 us, 8192 x 8192 1664 -> 1258 us.
+// Per cell about 560 thread instructions in the predictor and 495 in the
+// corrector with 4 rows per warp, 511 and 451 with 8 (865 and 800 with a cell
+// per thread and the fluxes in shared memory).  128 registers, no spills, 4
+// blocks of 128 threads per SM: at 16 warps per SM it is bound by the latency
+// of its own chains (0.64 of the issue slots with 4 rows per warp, 0.57 with
+// 8).  Mean of both stages, with events around the launches: 2048 x 2048 cells
+// 115 -> 93 us, 8192 x 8192 1664 -> 1299 us.
 #pragma once
 #include "celeris_internal.cuh"
 #include "celeris_physics.cuh"
