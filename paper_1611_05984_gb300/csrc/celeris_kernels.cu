@@ -825,18 +825,18 @@ __device__ __forceinline__ void stencil_tile(const StencilArgs<real> &A, const O
         } else {
             F = fma(mul_r(hb, -C.hgx), sx, div(1));
             Gq = fma(mul_r(hb, -C.hgy), sy, div(2));
-        }
-        if (sizeof(real) == 8 && friction != kFricNone) {   // Eq. 31-32 with the Eq. 14 device
-            const real fm = mul_r(friction_depth(friction, C.fric, hb, eps, C.hwet),
-                                  sqrt_r(fma(P0, P0, mul_r(Q0, Q0))));
-            F = fma(-fm, P0, F);
-            Gq = fma(-fm, Q0, Gq);
+            if (friction != kFricNone) {   // Eq. 31-32 with the Eq. 14 device
+                const real fm = mul_r(friction_depth(friction, C.fric, hb, eps, C.hwet),
+                                      sqrt_r(fma(P0, P0, mul_r(Q0, Q0))));
+                F = fma(-fm, P0, F);
+                Gq = fma(-fm, Q0, Gq);
+            }
         }
         real Fs = real(0), Gs = real(0);
         const int od = (cy + 1) * kDStride + cx + 1;
         const real dd = sm.d[od];
-        if (sizeof(real) == 4 && bsnq) {
-            if constexpr (sizeof(real) == 4) {
+        if constexpr (sizeof(real) == 4) {
+            if (bsnq) {
                 constexpr int S1 = kStride;
                 const real ddx = mul2(sub2(sm.d[od + 1], sm.d[od - 1]), kc<real>(A, kcHrdx));
                 const real ddy = mul2(sub2(sm.d[od + kDStride], sm.d[od - kDStride]), kc<real>(A, kcHrdy));
